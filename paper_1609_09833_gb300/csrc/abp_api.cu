@@ -164,6 +164,8 @@ struct abp_ctx {
   size_t hill_cap = 0;
   KernelTimer *timer = nullptr;  // ABP_TUNE_TIMING
   std::mutex mu;
+  cudaMemPool_t pool = nullptr;  // scratch of calls (struct Scratch)
+  std::mutex pool_mu;
 };
 
 struct abp_grid {
@@ -192,6 +194,52 @@ struct abp_walker {
 };
 
 namespace {
+
+constexpr size_t kPoolKeep = 256u << 20;     // bytes a context's scratch pool keeps between calls
+constexpr size_t kReadoutChunk = 32u << 20;  // staging bytes of a readout
+
+// Scratch of one call, ordered on the context's stream: taken from the
+// context's own memory pool (made at its first use, which keeps up to
+// kPoolKeep bytes between calls and is given back with the context) and
+// returned to it when the object goes out of scope, behind the work queued
+// so far. Calls on different streams or threads never share a block, and
+// under stream capture the block belongs to the graph. p is null if there is
+// no memory (err says why).
+struct Scratch {
+  void *p = nullptr;
+  cudaError_t err = cudaSuccess;
+  cudaStream_t st;
+  Scratch(abp_ctx *ctx, size_t bytes) : st(ctx->stream) {
+    cudaMemPool_t pool = nullptr;
+    {
+      std::lock_guard<std::mutex> lk(ctx->pool_mu);
+      if (!ctx->pool) {
+        cudaMemPoolProps pr{};
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = ctx->device;
+        uint64_t keep = kPoolKeep;
+        err = cudaMemPoolCreate(&ctx->pool, &pr);
+        if (err == cudaSuccess) err = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (err != cudaSuccess && ctx->pool) {
+          cudaMemPoolDestroy(ctx->pool);
+          ctx->pool = nullptr;
+        }
+      }
+      pool = ctx->pool;
+    }
+    if (pool) err = cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), pool, st);
+    if (err != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  ~Scratch() {
+    if (p) cudaFreeAsync(p, st);
+  }
+  Scratch(const Scratch &) = delete;
+  Scratch &operator=(const Scratch &) = delete;
+};
 
 abp_status set_device(const abp_ctx *ctx) {
   int cur = -1;
@@ -460,6 +508,7 @@ void abp_ctx_destroy(abp_ctx *ctx) {
   if (ctx->log.rec) cudaFree(ctx->log.rec);
   if (ctx->log.count) cudaFree(ctx->log.count);
   if (ctx->ctr) cudaFree(ctx->ctr);
+  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   delete ctx->timer;
   delete ctx;
 }
@@ -1593,45 +1642,53 @@ abp_status abp_grid_restore(abp_ctx *ctx, abp_grid *g, const void *src, int src_
   return ABP_OK;
 }
 
+// abp_bias_readout where the device has no memory left for the staging block:
+// the records to the host, converted there.
+static abp_status readout_by_host(abp_ctx *ctx, const abp_grid *g, void *dst, int dst_is_device, int dtype) {
+  const GridDev &gd = g->g;
+  const int nf = 1 + gd.d, comp = gd.d == 1 ? 2 : 4;
+  std::vector<unsigned char> raw(g->bytes);
+  CUDA_TRY(cudaMemcpyAsync(raw.data(), gd.rec, g->bytes, cudaMemcpyDeviceToHost, ctx->stream));
+  CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  std::vector<unsigned char> out((size_t)gd.nodes * nf * (dtype == ABP_F64 ? 8 : 4));
+  for (long long i = 0; i < gd.nodes; ++i)
+    for (int q = 0; q < nf; ++q) {
+      const unsigned char *r = raw.data() + (size_t)i * gd.rec_bytes;
+      const float *f = reinterpret_cast<const float *>(r);
+      const double x = gd.prec == ABP_PREC_FP32_COMP ? (double)f[q] + (double)f[comp + q]
+                                                     : reinterpret_cast<const double *>(r)[q];
+      const size_t j = (size_t)i * nf + q;
+      if (dtype == ABP_F64)
+        reinterpret_cast<double *>(out.data())[j] = x;
+      else
+        reinterpret_cast<float *>(out.data())[j] = (float)x;
+    }
+  if (dst_is_device)
+    CUDA_TRY(cudaMemcpy(dst, out.data(), out.size(), cudaMemcpyHostToDevice));
+  else
+    std::memcpy(dst, out.data(), out.size());
+  return ABP_OK;
+}
+
 abp_status abp_bias_readout(abp_ctx *ctx, const abp_grid *g, void *dst, int dst_is_device, int dtype) {
   if (!ctx || !g || !dst || g->ctx != ctx) return fail(ABP_ERR_INVALID_ARG, "bad argument");
   if (dtype != ABP_F32 && dtype != ABP_F64) return fail(ABP_ERR_INVALID_ARG, "bad dtype");
   abp_status st = set_device(ctx);
   if (st) return st;
+  // converted on the device into a staging block, copied from there (the copy
+  // checks the destination as it always did: its kind, size and alignment)
   const GridDev &gd = g->g;
-  const int d = gd.d, nf = 1 + d;
-  std::vector<unsigned char> raw(g->bytes);
-  CUDA_TRY(cudaMemcpyAsync(raw.data(), gd.rec, g->bytes, cudaMemcpyDeviceToHost, ctx->stream));
+  const size_t node = (size_t)(1 + gd.d) * (dtype == ABP_F64 ? 8 : 4);
+  const long long chunk = std::min(gd.nodes, (long long)(kReadoutChunk / node));
+  Scratch stage(ctx, (size_t)chunk * node);
+  if (!stage.p) return readout_by_host(ctx, g, dst, dst_is_device, dtype);
+  for (long long i = 0; i < gd.nodes; i += chunk) {
+    const long long c = std::min(chunk, gd.nodes - i);
+    CUDA_TRY(launch_readout(gd, i, c, stage.p, dtype == ABP_F64, ctx->stream));
+    CUDA_TRY(cudaMemcpyAsync(static_cast<unsigned char *>(dst) + (size_t)i * node, stage.p, (size_t)c * node,
+                             dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream));
+  }
   CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-  const size_t nvals = (size_t)gd.nodes * nf;
-  std::vector<double> v(nvals);
-  for (long long i = 0; i < gd.nodes; ++i) {
-    for (int q = 0; q < nf; ++q) {
-      double x;
-      if (gd.prec == ABP_PREC_FP32_COMP) {
-        const float *r = reinterpret_cast<const float *>(raw.data() + (size_t)i * gd.rec_bytes);
-        int comp_off = d == 1 ? 2 : 4;
-        x = (double)r[q] + (double)r[comp_off + q];
-      } else {
-        x = reinterpret_cast<const double *>(raw.data() + (size_t)i * gd.rec_bytes)[q];
-      }
-      v[(size_t)i * nf + q] = x;
-    }
-  }
-  const void *src = v.data();
-  std::vector<float> vf;
-  size_t bytes = nvals * sizeof(double);
-  if (dtype == ABP_F32) {
-    vf.resize(nvals);
-    for (size_t i = 0; i < nvals; ++i) vf[i] = (float)v[i];
-    src = vf.data();
-    bytes = nvals * sizeof(float);
-  }
-  if (dst_is_device) {
-    CUDA_TRY(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice));
-  } else {
-    std::memcpy(dst, src, bytes);
-  }
   return ABP_OK;
 }
 

@@ -166,4 +166,8 @@ cudaError_t smem_attr(const void *fn, size_t bytes);
 cudaError_t launch_deliver(const TableEntry *table, int nw, void *forces, const long long *foff, int mode, int fp64,
                            cudaStream_t st);
 
+// Node records [first, first + count) as fields [count][1 + d] (FP64 or FP32) at `out` (device).
+cudaError_t launch_readout(const GridDev &gd, long long first, long long count, void *out, int fp64_out,
+                           cudaStream_t st);
+
 }  // namespace abp
