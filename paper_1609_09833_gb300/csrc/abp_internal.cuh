@@ -169,7 +169,7 @@ constexpr int kAtomTerms = 2 * kMaxCv;  // per atom: up to 2 list entries per CV
 // ~1.2e-7 rad near +-pi, would otherwise move the hill by 2e-6 of its width
 // or more, against a 1e-5 tolerance on the grid fields.
 constexpr double kDihedralHpWidth = 0.06;
-constexpr int kMabpBoxBytes = 96 * 1024;  // windowed mABP: the union of a window's stencil boxes, at most
+constexpr int kMabpUnion = 8192;  // windowed mABP: nodes of the union of a window's stencil boxes, at most
 constexpr int kWinBytes = 64 * 1024;    // its coordinate double buffer, at most
 constexpr int kWtBoxBytes = 64 * 1024;  // windowed WT: a deposit's stencil box, at most
 
@@ -203,8 +203,7 @@ __host__ __device__ inline int window_steps(int natoms, const CvDev *cv, int d, 
 //   cn        per COORD CV: dCN/dx per list entry and per-warp partials
 //   tile      optional copy of a box of the walker's grid (node records); in
 //             the windowed form, a deposit's stencil box (WT walkers of 1 or 2
-//             CVs whose box has at most one node per chain-half thread) or
-//             the union of a window's boxes (mABP)
+//             CVs whose box has at most one node per chain-half thread)
 struct GroupLayout {
   int xs0, xs1, fs, steps, atoms, lists, cn, tile, total;
   int win, xstride;  // windowed form: steps per window (0 = per-step form), row stride in records
@@ -280,9 +279,7 @@ __host__ __device__ inline GroupLayout group_layout(int natoms, const CvDev *cv,
   if (L.win) {
     for (int k = 0; k < 3; ++k) L.T[k] = 0;
     L.tile_nodes = 0;
-    if (mabp) {
-      L.box = kMabpBoxBytes;
-    } else {
+    if (!mabp) {
       // only a box the chain half can hold one node per thread of
       // (the window's single-round chain); larger boxes go round by round
       long long nodes = 1;

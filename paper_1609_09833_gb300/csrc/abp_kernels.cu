@@ -259,11 +259,6 @@ __device__ __forceinline__ float4 lds128(unsigned a) {
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
   return v;
 }
-__device__ __forceinline__ void sts128(unsigned a, const float4 &v) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-               : "memory");
-}
-
 // Deposit steps of a window (bit j: step t0 + j).
 __device__ __forceinline__ unsigned window_dmask(long long step0, int t0, int nt, long long stride) {
   const long long rem = (step0 + t0) % stride;
@@ -326,7 +321,7 @@ struct WindowCtx {
   int W, nwin, mode;
   bool serial_out;
   unsigned long long stream;
-  unsigned char *box;    // a deposit's stencil box (WT) or the union of a window's boxes (mABP); NULL: none
+  unsigned char *box;    // a WT deposit's stencil box; NULL: none
 
   __device__ __forceinline__ int nt_of(int w) const { return min(W, nsteps - w * W); }
   __device__ __forceinline__ StepRec<Real> *steps_of(int w) const { return steps + (w % 3) * W; }
@@ -418,7 +413,7 @@ struct WindowCtx {
   template <int UNR, int DIM>
   __device__ __forceinline__ void chain(const Grp &g, int w) const {
     if (fx->wd.method == ABP_METHOD_MABP) {
-      if (box && chain_mabp<DIM>(g, w)) return;
+      if (chain_mabp<DIM>(g, w)) return;
     } else if constexpr (DIM < 3) {
       if (box && chain_one<DIM>(g, w)) return;
     }
@@ -523,27 +518,35 @@ struct WindowCtx {
     return true;
   }
 
-  // mABP: the window's deposits through shared memory. Every hill has the
-  // fixed height w and sits on its step's nearest node, so no deposit depends
-  // on a look-up: the union of the window's stencil boxes is copied into
-  // shared memory, the hills are applied there one after another (the same
-  // compensated additions as chain_seq's, so the same bits), each step reads
-  // its node there once the hills up to its own are in, and the box is
-  // written back. Steps whose node lies outside the union read the grid.
-  // Returns false (nothing done) when the union does not fit.
+  // mABP: a window's deposits node by node. Every hill has the fixed height w
+  // and sits on its step's nearest node, so no deposit depends on a look-up:
+  // each thread takes NB nodes of the union of the window's stencil boxes
+  // into registers, walks the window's steps in order, adds each hill that
+  // covers its node (the same compensated additions as chain_seq's in the
+  // same order per node, so the same bits), leaves a step's raw histograms
+  // in its record where its node is the step's look-up node, and stores the
+  // nodes once. No barrier between hills. Steps whose node lies outside the
+  // union read the grid. Bound by the instructions per (node, hill) of the
+  // chain half's warps (23 x 23 nodes x 32 hills x ~40 on four warps). Two
+  // RMSD CVs on 480 x 480, 441-node hills, 64 walkers x 1000 steps: 1.55 ms
+  // with a box in shared memory and a barrier per hill, 1.01 ms now.
+  // Returns false (nothing done) for a union of more than kMabpUnion nodes:
+  // there the nodes no hill covers cost more than chain_seq's barriers.
   template <int DIM>
   __device__ bool chain_mabp(const Grp &g, int w) const {
     const WalkerDev &wd = fx->wd;
     const GridDev &gd = wd.g;
-    constexpr int d = DIM;
-    const int nt = nt_of(w), t0 = w * W, rb = gd.rec_bytes;
+    constexpr int d = DIM, rb = DIM > 1 ? 32 : 16;
+    constexpr int NB = sizeof(Real) == 4 ? 5 : 3;
+    const int nt = nt_of(w), t0 = w * W;
     StepRec<Real> *st = steps_of(w);
     const unsigned bad = fx->winbad[w % 3];
     const unsigned gdep = window_dmask(step0, t0, nt, wd.stride) & ~bad;
-    const int first = gdep ? __ffs(gdep) - 1 : nt;
     int org[3] = {0, 0, 0}, span[3] = {1, 1, 1};
     long long nodes = gdep ? 1 : 0;
     if (gdep) {
+      const int first = __ffs(gdep) - 1;
+#pragma unroll
       for (int k = 0; k < d; ++k) {
         const int n = gd.n[k], c0 = st[first].da[k];
         int lo = 0, hi = 0;
@@ -573,48 +576,18 @@ struct WindowCtx {
         }
         nodes *= span[k];
       }
-      if (nodes * rb > kMabpBoxBytes) return false;
+      if (nodes > kMabpUnion) return false;
     }
-    // box index of a node, or -1 outside the box
-    auto box_index = [&](const int *j) -> int {
-      int idx = 0, mul = 1;
+    // is node j inside the union?
+    auto inside = [&](const int *j) -> bool {
+#pragma unroll
       for (int k = 0; k < d; ++k) {
         int r = j[k] - org[k];
         if (gd.periodic[k] && r < 0) r += gd.n[k];
-        if (r < 0 || r >= span[k]) return -1;
-        idx += mul * r;
-        mul *= span[k];
+        if (r < 0 || r >= span[k]) return false;
       }
-      return idx;
+      return true;
     };
-    // raw histograms of a step's node, kept in V / dv until the window's end
-    auto raw_copy = [&](StepRec<Real> &s, const unsigned char *p) {
-      Real v[4] = {0, 0, 0, 0};
-      float4 ra, rbv;
-      rec_load<DIM>(p, ra, rbv);
-      rec_vals<Real, DIM>(ra, rbv, v);
-      s.V = v[0];
-      for (int k = 0; k < 3; ++k) s.dv[k] = v[1 + k];
-    };
-    const unsigned char *rec = reinterpret_cast<const unsigned char *>(gd.rec);
-    auto node_ptr = [&](int idx) -> const unsigned char * {
-      long long node = 0, mul = 1;
-      int r = idx;
-      for (int k = 0; k < d; ++k) {
-        const int q = r % span[k];
-        r /= span[k];
-        int j = org[k] + q;
-        if (j >= gd.n[k]) j -= gd.n[k];
-        node += mul * j;
-        mul *= gd.n[k];
-      }
-      return rec + chk_node(gd, node) * rb;
-    };
-    // steps read from the box (bit j), the rest from the grid
-    unsigned inbox = 0;
-    if (gdep)
-      for (int j = 0; j < nt; ++j)
-        if (!((bad >> j) & 1) && box_index(st[j].da) >= 0) inbox |= 1u << j;
     // tables of the node-centred hill (the same for every deposit)
     if (g.t < d) {
       fx->da[g.t] = 0;
@@ -623,85 +596,119 @@ struct WindowCtx {
     }
     g.sync();
     build_tables<Real>(g, fx);
-    // the box in; steps outside it read the grid
-    for (int i = g.t; i < nodes; i += g.G) {
-      const float4 *src = reinterpret_cast<const float4 *>(node_ptr(i));
-      float4 *dst = reinterpret_cast<float4 *>(box + (size_t)i * rb);
-      dst[0] = src[0];
-      if (rb == 32) dst[1] = src[1];
-    }
+    // steps outside the union read the grid (before and after the window's
+    // hills alike); the others are met in the walk below
+    unsigned inbox = 0;
+    if (gdep)
+      for (int j = 0; j < nt; ++j)
+        if (!((bad >> j) & 1) && inside(st[j].da)) inbox |= 1u << j;
     for (int j = g.t; j < nt; j += g.G)
       if (!((bad >> j) & 1) && !((inbox >> j) & 1)) interp_one<Real, DIM>(wd, st[j]);
-    g.sync();
-    for (int j = g.t; j < first; j += g.G)
-      if ((inbox >> j) & 1) raw_copy(st[j], box + (size_t)box_index(st[j].da) * rb);
+    g.sync();  // the tables
+    // axis 0's factors times the hill height, and each step's first stencil
+    // node relative to the union's origin (on a periodic axis in [0, n); the
+    // node indexes build_tables left in tabJ are not used here)
     const Real h = (Real)wd.w;
-    const int s0 = 2 * wd.R[0] + 1, s1 = d > 1 ? 2 * wd.R[1] + 1 : 1, s2 = d > 2 ? 2 * wd.R[2] + 1 : 1;
-    const int sp01 = s0 * s1;
-    for (unsigned m = gdep; m; m &= m - 1) {
-      const int j = __ffs(m) - 1;
-      const unsigned rest = m & (m - 1);
-      const int next = rest ? __ffs(rest) - 1 : nt;
-      g.sync();  // the hills and look-ups before this hill are done
-      // box-relative position of the hill's first node, per axis
-      // (on a periodic axis taken into [0, n), so that one wrap suffices below)
-      int base[3] = {0, 0, 0};
-      for (int k = 0; k < d; ++k) {
-        base[k] = st[j].da[k] - wd.R[k] - org[k];
-        if (gd.periodic[k]) base[k] = ((base[k] % gd.n[k]) + gd.n[k]) % gd.n[k];
-      }
-      const bool centre_in = (inbox >> j) & 1;
-      // stencil positions (o0 fastest), advanced without division
-      Iter2 it(g.t, g.G, s0);
-      for (int idx = g.t; idx < sp01 * s2; idx += g.G, it.next()) {
-        const int o0 = it.i, o12 = it.j, o1 = d > 2 ? o12 % s1 : o12, o2 = d > 2 ? o12 / s1 : 0;
-        const int o[3] = {o0, o1, o2};
-        int bi = 0, mul = 1;
-        bool in = true;
-        for (int k = 0; k < d; ++k) {
-          const int n = gd.n[k];
-          int r = base[k] + o[k];  // node - org
-          if (gd.periodic[k]) {
-            if (r >= n) r -= n;
-          } else {
-            const int jn = r + org[k];
-            in = in && jn >= 0 && jn < n;
-          }
-          in = in && r >= 0 && r < span[k];
-          bi += mul * r;
-          mul *= span[k];
-        }
-        if (!in) continue;
-        Real G = h * fx->tabG[0][o0];
-        if (d > 1) G = G * fx->tabG[1][o1];
-        if (d > 2) G = G * fx->tabG[2][o2];
-        const Real d0 = fx->tabD[0][o0], d1 = d > 1 ? fx->tabD[1][o1] : (Real)0,
-                   d2 = d > 2 ? fx->tabD[2][o2] : (Real)0;
-        unsigned char *p = box + (size_t)bi * rb;
-        // the record through shared-memory loads and stores
-        const unsigned sa = (unsigned)__cvta_generic_to_shared(p);
-        float4 ra = lds128(sa), rbv = rb == 32 ? lds128(sa + 16) : make_float4(0, 0, 0, 0);
-        rmw_regs<Real>(d, ra, rbv, G, d0, d1, d2);
-        sts128(sa, ra);
-        if (rb == 32) sts128(sa + 16, rbv);
-        // the hill's own step reads its centre right after it
-        if (centre_in && o0 == wd.R[0] && (d < 2 || o1 == wd.R[1]) && (d < 3 || o2 == wd.R[2])) raw_copy(st[j], p);
-      }
-      if (g.t == g.G - 1 && log.rec) window_height<Real, DIM>(fx, st[j], step0 + t0 + j, log);
-      if (next > j + 1) {  // steps between this hill and the next read after it
-        g.sync();
-        for (int q = j + 1 + g.t; q < next; q += g.G)
-          if ((inbox >> q) & 1) raw_copy(st[q], box + (size_t)box_index(st[q].da) * rb);
-      }
+    for (int o = g.t; o < 2 * wd.R[0] + 1; o += g.G) fx->tabG[0][o] = mul_rn(h, fx->tabG[0][o]);
+    for (int i = g.t; i < nt * d; i += g.G) {
+      const int k = i % d, j = i / d;
+      int b = st[j].da[k] - wd.R[k] - org[k];
+      if (gd.periodic[k]) b = ((b % gd.n[k]) + gd.n[k]) % gd.n[k];
+      fx->tabJ[k][j] = b;
     }
     g.sync();
-    // the box out; the raw histograms of the steps read in it become the bias
-    for (int i = g.t; i < nodes; i += g.G) {
-      float4 *dst = reinterpret_cast<float4 *>(const_cast<unsigned char *>(node_ptr(i)));
-      const float4 *src = reinterpret_cast<const float4 *>(box + (size_t)i * rb);
-      dst[0] = src[0];
-      if (rb == 32) dst[1] = src[1];
+    unsigned char *rec = reinterpret_cast<unsigned char *>(gd.rec);
+    // the walk's constants in registers: half-widths, and the wrap of a
+    // periodic axis (0 on others, where a node below the stencil stays below)
+    int R[DIM], wrap[DIM];
+#pragma unroll
+    for (int k = 0; k < d; ++k) {
+      R[k] = wd.R[k];
+      wrap[k] = gd.periodic[k] ? gd.n[k] : 0;
     }
+    for (int i0 = g.t; i0 < nodes; i0 += NB * g.G) {
+      float4 ra[NB], rbv[NB];
+      int q[NB][DIM];
+      unsigned char *ptr[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        int r = i0 + u * g.G;
+        ptr[u] = nullptr;
+        ra[u] = rbv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < nodes) {
+          long long node = 0, mul = 1;
+#pragma unroll
+          for (int k = 0; k < d; ++k) {
+            q[u][k] = r % span[k];
+            r /= span[k];
+            int j = org[k] + q[u][k];
+            if (j >= gd.n[k]) j -= gd.n[k];
+            node += mul * j;
+            mul *= gd.n[k];
+          }
+          ptr[u] = rec + chk_node(gd, node) * rb;
+          rec_load<DIM>(ptr[u], ra[u], rbv[u]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < d; ++k) q[u][k] = -(1 << 29);  // in no stencil
+        }
+      }
+      for (int j = 0; j < nt; ++j) {
+        if (!((inbox >> j) & 1)) continue;  // neither deposits nor is read here (a deposit's centre is inside)
+        const bool dep = (gdep >> j) & 1;
+        int b[DIM];
+#pragma unroll
+        for (int k = 0; k < d; ++k) b[k] = fx->tabJ[k][j];
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+          int o[3] = {0, 0, 0};
+          bool in = true, centre = true;
+#pragma unroll
+          for (int k = 0; k < d; ++k) {
+            int r = q[u][k] - b[k];
+            r += r < 0 ? wrap[k] : 0;
+            in = in & ((unsigned)r <= (unsigned)(2 * R[k]));
+            centre = centre & (r == R[k]);
+            o[k] = r;
+          }
+          if (dep) {
+            // a hill that misses the node leaves the record as it was
+#pragma unroll
+            for (int k = 0; k < d; ++k) o[k] = in ? o[k] : 0;
+            Real G = fx->tabG[0][o[0]];
+            if (d > 1) G = mul_rn(G, fx->tabG[1][o[1]]);
+            if (d > 2) G = mul_rn(G, fx->tabG[2][o[2]]);
+            float4 na = ra[u], nb = rbv[u];
+            rmw_regs<Real>(d, na, nb, G, fx->tabD[0][o[0]], d > 1 ? fx->tabD[1][o[1]] : (Real)0,
+                           d > 2 ? fx->tabD[2][o[2]] : (Real)0);
+            if (in) {
+              ra[u] = na;
+              rbv[u] = nb;
+            }
+          }
+          if (in && centre) {  // the step's look-up: its raw histograms, turned into the bias below
+            Real v[4] = {0, 0, 0, 0};
+            rec_vals<Real, DIM>(ra[u], rbv[u], v);
+            st[j].V = v[0];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) st[j].dv[k] = v[1 + k];
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+        if (ptr[u]) {
+          float4 *p = reinterpret_cast<float4 *>(ptr[u]);
+          p[0] = ra[u];
+          if (rb == 32) p[1] = rbv[u];
+        }
+    }
+    if (g.t == g.G - 1 && log.rec)
+      for (unsigned m = gdep; m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        window_height<Real, DIM>(fx, st[j], step0 + t0 + j, log);
+      }
+    g.sync();
     for (int j = g.t; j < nt; j += g.G)
       if ((inbox >> j) & 1) {
         Real acc[4] = {st[j].V, st[j].dv[0], st[j].dv[1], st[j].dv[2]};
