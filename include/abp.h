@@ -182,6 +182,8 @@ abp_status abp_ctx_bytes(const abp_ctx *ctx, size_t *used, size_t *budget);
  *   ABP_TUNE_TILE            1 = give groups a shared-memory tile of their
  *                            grid when it fits (launches of >= 8 steps),
  *                            0 or -1 = never (the default)
+ *   (Any of the first three set, or LEAN, keeps abp_run in the forms with a
+ *   group per walker.)
  *   ABP_TUNE_LEAN            1 = FP32 launches without a tile use the
  *                            kernel compiled for 128 registers per thread
  *                            (two 256-thread CTAs per SM), 0 = the default
@@ -242,9 +244,12 @@ abp_status abp_step(abp_ctx *ctx, abp_walker *const *walkers, int n, const void 
 abp_status abp_forces(abp_ctx *ctx, abp_walker *const *walkers, int n, void *forces_dev, int forces_dtype,
                       const int64_t *force_offsets_dev, int mode);
 
-/* The fused batched form: nsteps consecutive MD steps step0..step0+nsteps-1
- * of n walkers with their own grids in one launch, equal per step and walker
- * to abp_step followed by abp_forces. Coordinates of step t at record
+/* The batched form: nsteps consecutive MD steps step0..step0+nsteps-1 of n
+ * walkers with their own grids, equal per step and walker to abp_step followed
+ * by abp_forces. One launch for short calls; longer ones run in three launches
+ * over scratch of at most 240 MB from a pool that the library keeps per device
+ * while it has contexts there (without that memory, one launch: the same
+ * results). Coordinates of step t at record
  * coord_offsets_dev[w] + t * coord_step_stride + i; forces written (by mode)
  * at force_offsets_dev[w] + t * force_step_stride + i. Walkers that share a
  * grid are rejected (use abp_step). */

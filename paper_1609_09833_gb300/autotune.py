@@ -34,7 +34,8 @@ def signature(specs, nsteps: int) -> str:
 
 def candidates(specs):
     cn = any(c["type"] == "coord" for s in specs for c in s["cvs"])
-    out = []
+    # the library's own choice (the split form for calls of several steps)
+    out = [{"group_threads": 0, "groups_per_cta": 0, "tile": -1, "lean": 0}]
     for G in ((64, 128, 256) if cn else (32, 64, 128, 256)):
         for gpc in ((1, 2) if G >= 128 else (1, 2, 4)):
             for lean in (0, 1):

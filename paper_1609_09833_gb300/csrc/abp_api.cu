@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -164,8 +165,6 @@ struct abp_ctx {
   size_t hill_cap = 0;
   KernelTimer *timer = nullptr;  // ABP_TUNE_TIMING
   std::mutex mu;
-  cudaMemPool_t pool = nullptr;  // scratch of calls (struct Scratch)
-  std::mutex pool_mu;
 };
 
 struct abp_grid {
@@ -195,40 +194,68 @@ struct abp_walker {
 
 namespace {
 
-constexpr size_t kPoolKeep = 256u << 20;     // bytes a context's scratch pool keeps between calls
+constexpr size_t kPoolKeep = 256u << 20;     // bytes the scratch pool of a device keeps between calls
 constexpr size_t kReadoutChunk = 32u << 20;  // staging bytes of a readout
 
+// The library's memory pool of a device, shared by its contexts there: made
+// by the first call that needs scratch, given back with the last context. It
+// keeps up to kPoolKeep bytes between calls (mapping them again on every call
+// took ~0.3 ms).
+constexpr int kMaxDevices = 64;
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  int contexts = 0;
+};
+std::mutex g_pool_mu;
+DevicePool g_pools[kMaxDevices];
+
+void pool_context(int device, int delta) {
+  if (device < 0 || device >= kMaxDevices) return;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  DevicePool &p = g_pools[device];
+  p.contexts += delta;
+  if (p.contexts == 0 && p.pool) {
+    cudaMemPoolDestroy(p.pool);
+    p.pool = nullptr;
+  }
+}
+
+cudaError_t pool_get(int device, cudaMemPool_t *out) {
+  *out = nullptr;
+  if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  DevicePool &p = g_pools[device];
+  cudaError_t e = cudaSuccess;
+  if (!p.pool) {
+    cudaMemPoolProps pr{};
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    pr.location.id = device;
+    uint64_t keep = kPoolKeep;
+    e = cudaMemPoolCreate(&p.pool, &pr);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess && p.pool) {
+      cudaMemPoolDestroy(p.pool);
+      p.pool = nullptr;
+    }
+  }
+  *out = p.pool;
+  return e;
+}
+
 // Scratch of one call, ordered on the context's stream: taken from the
-// context's own memory pool (made at its first use, which keeps up to
-// kPoolKeep bytes between calls and is given back with the context) and
-// returned to it when the object goes out of scope, behind the work queued
-// so far. Calls on different streams or threads never share a block, and
-// under stream capture the block belongs to the graph. p is null if there is
-// no memory (err says why).
+// device's pool and returned to it when the object goes out of scope, behind
+// the work queued so far. Calls on different streams or threads never share a
+// block, and under stream capture the block belongs to the graph. p is null
+// if there is no memory (err says why).
 struct Scratch {
   void *p = nullptr;
   cudaError_t err = cudaSuccess;
   cudaStream_t st;
   Scratch(abp_ctx *ctx, size_t bytes) : st(ctx->stream) {
     cudaMemPool_t pool = nullptr;
-    {
-      std::lock_guard<std::mutex> lk(ctx->pool_mu);
-      if (!ctx->pool) {
-        cudaMemPoolProps pr{};
-        pr.allocType = cudaMemAllocationTypePinned;
-        pr.location.type = cudaMemLocationTypeDevice;
-        pr.location.id = ctx->device;
-        uint64_t keep = kPoolKeep;
-        err = cudaMemPoolCreate(&ctx->pool, &pr);
-        if (err == cudaSuccess) err = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (err != cudaSuccess && ctx->pool) {
-          cudaMemPoolDestroy(ctx->pool);
-          ctx->pool = nullptr;
-        }
-      }
-      pool = ctx->pool;
-    }
-    if (pool) err = cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), pool, st);
+    err = pool_get(ctx->device, &pool);
+    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), pool, st);
     if (err != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
@@ -446,6 +473,7 @@ abp_status abp_ctx_create(abp_ctx **out, int device, void *cuda_stream, size_t h
     delete c;
     return st;
   }
+  pool_context(device, 1);
   *out = c;
   return ABP_OK;
 }
@@ -508,7 +536,7 @@ void abp_ctx_destroy(abp_ctx *ctx) {
   if (ctx->log.rec) cudaFree(ctx->log.rec);
   if (ctx->log.count) cudaFree(ctx->log.count);
   if (ctx->ctr) cudaFree(ctx->ctr);
-  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  pool_context(ctx->device, -1);
   delete ctx->timer;
   delete ctx;
 }
@@ -1093,6 +1121,63 @@ static abp_status big_items(abp_ctx *ctx, const std::vector<abp_walker *> &ws, c
   return ABP_OK;
 }
 
+// The split form of a batch (abp_split.cu), in blocks of walkers and steps
+// whose records fit the call's scratch. *done is false, with nothing run, if
+// there is no memory for it.
+constexpr size_t kSplitScratch = 240u << 20;  // (below kPoolKeep, so that the pool keeps it)
+static abp_status run_split(abp_ctx *ctx, const std::vector<abp_walker *> &ws, const TableEntry *table, bool win,
+                            SplitArgs a, int nsteps, bool *done) {
+  SplitShape shape;
+  int jrec = 0, max_atoms = 0;
+  size_t words = 0;
+  for (const abp_walker *w : ws) {
+    split_shape(w->hd, win, &shape);
+    if (!win) {
+      jrec = std::max(jrec, split_jac_records(w->hd));
+      words = std::max(words, (size_t)split_term_words(w->hd));
+    }
+    max_atoms = std::max(max_atoms, w->hd.natoms);
+  }
+  a.serial = a.forces && std::llabs(a.fstride) < max_atoms;
+  a.jstride = jrec;
+  a.term_stride = words;
+  // per walker and step its record and gradient records, per walker its atoms' terms
+  const size_t item = split_step_bytes() + (size_t)jrec * 16, fixed = words * 8;
+  const size_t nb = std::max<size_t>(1, std::min(ws.size(), kSplitScratch / (item + fixed)));
+  const size_t room = kSplitScratch > nb * fixed ? kSplitScratch - nb * fixed : 0;
+  long long T = (long long)std::max<size_t>(1, room / (item * nb));
+  T = std::min<long long>(std::min(T, 200000ll), nsteps);  // (grid dimensions of at most 65535)
+  if (T > 32) T -= T < nsteps ? T % 32 : 0;
+  const size_t recs = (nb * (size_t)T * split_step_bytes() + 255) / 256 * 256, jac = nb * (size_t)T * jrec * 16;
+  Scratch mem(ctx, recs + jac + nb * fixed);
+  *done = mem.p != nullptr;
+  if (!mem.p) return ABP_OK;
+  unsigned char *m = static_cast<unsigned char *>(mem.p);
+  a.recs = m;
+  a.jac = m + recs;
+  a.terms = words ? m + recs + jac : nullptr;
+  for (size_t w = 0; w < ws.size(); w += nb) {
+    a.table = table + w;
+    a.nw = (int)std::min(nb, ws.size() - w);
+    for (long long t = 0; t < nsteps; t += T) {
+      a.t0 = t;
+      a.nsteps = (int)std::min<long long>(T, nsteps - t);
+      a.last = t + T >= nsteps;
+      cudaError_t e = launch_split(a, shape, ctx->sms, ctx->timer, ctx->stream);
+      if (e != cudaSuccess) return fail(ABP_ERR_CUDA, "split launch: %s", cudaGetErrorString(e));
+    }
+  }
+  return ABP_OK;
+}
+
+// Steps from which a batch of windowed-form walkers takes the split form: its
+// three launches cost ~25 us where the group form's one costs ~18 us and then
+// 0.2 us a step (well-tempered) or 1 us a step (mABP), each again per round of
+// walkers over the SMs. Measured, split / group, us: 64 walkers 32 steps 28 /
+// 23, 64 steps 31 / 31, 256 steps 50 / 66; 300 walkers 16 steps 27 / 37; mABP
+// 16 steps 27 / 29.
+int split_min_steps(int n, int sms, bool mabp) { return n > sms || mabp ? 16 : 64; }
+
 static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, const void *coords, int cdt,
                              const int64_t *coff, int64_t cstride, void *forces, const int64_t *foff,
                              int64_t fstride, int mode, int64_t step0, int nsteps) {
@@ -1142,6 +1227,30 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     if (lw.empty()) continue;
     RunArgs a{};
     if ((st = sub_table(ctx, lw, li, &a.table))) return st;
+    // the split form (the same bits), unless a launch-shape knob asks for a
+    // group per walker or the call is too short for its three launches
+    bool mabp = true;
+    for (const abp_walker *w : lw) mabp = mabp && w->hd.method == ABP_METHOD_MABP;
+    bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1 &&
+                 (win ? nsteps >= split_min_steps((int)lw.size(), ctx->sms, mabp)
+                      : nsteps > 1 || (int)lw.size() > 2 * ctx->sms);
+    for (size_t i = 0; split && i < lw.size(); ++i) split = split_eligible(lw[i]->hd, win);
+    if (split) {
+      SplitArgs s{};
+      s.coords = coords;
+      s.coff = reinterpret_cast<const long long *>(coff);
+      s.cstride = cstride;
+      s.forces = forces;
+      s.foff = reinterpret_cast<const long long *>(foff);
+      s.fstride = fstride;
+      s.mode = mode;
+      s.step0 = step0;
+      s.log = ctx->log;
+      s.ctr = ctx->ctr;
+      bool done = false;
+      if ((st = run_split(ctx, lw, a.table, win, s, nsteps, &done))) return st;
+      if (done) continue;
+    }
     if ((st = pick_shape(ctx, lw.data(), (int)lw.size(), fp64, nsteps, win, &a.G, &a.groups_per_cta,
                          &a.group_bytes, &a.tile_budget)))
       return st;

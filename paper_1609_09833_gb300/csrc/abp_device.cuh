@@ -67,6 +67,17 @@ __device__ __forceinline__ unsigned long long l2_evict_first() {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// Rounded arithmetic with no contraction left to the compiler, so that every
+// inlined copy of a CV computes the same bits.
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // ---------------------------------------------------------------- groups
 
 struct Grp {
@@ -162,8 +173,9 @@ __device__ __forceinline__ bool grp_any(const Grp &g, GroupFixed<Real> *fx, int 
   return r != 0;
 }
 
-template <typename Real>
+template <typename Real, bool RN = false>
 __device__ __forceinline__ Real min_image(Real dx, double box, double inv_box) {
+  if constexpr (RN) return fma_rn(-(Real)box, floor(fma_rn(dx, (Real)inv_box, (Real)0.5)), dx);
   return dx - (Real)box * floor(dx * (Real)inv_box + (Real)0.5);
 }
 
@@ -314,68 +326,102 @@ __device__ __forceinline__ int com_finish_ff(const CvDev &c, const float *ra, co
   return ABP_WFLAG_SINGULAR;
 }
 
+// An FP32 COM distance by one warp: every weighted offset from the group's
+// first atom formed exactly as hi + lo (the difference x - r_G split by
+// two_sum, the product's error by fma; the tiny w times the difference's low
+// part rounded once) and summed with two_sum per lane; group A's three sums
+// then on lanes 0-15 and group B's on lanes 16-31, where each exchange level
+// adds the partner's high part with its exact error going to the low part;
+// finished in hi + lo (com_finish_ff). A group of hundreds of atoms spread
+// over nanometres would otherwise lose ~1e-7 nm, several millionths of a hill
+// a few grid spacings wide. The result is lane 0's.
+__device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, const int32_t *ib, const float *wa,
+                                            const float *wb, const float4 *xs, int lane, float &s, float &sl,
+                                            float *u) {
+  const float4 ra = xs[ia[0]], rb = xs[ib[0]];
+  float h[6] = {0, 0, 0, 0, 0, 0}, l[6] = {0, 0, 0, 0, 0, 0};
+  auto acc = [&](int q, float w, float x, float r) {
+    float dh, dl;
+    two_sum<float>(x, -r, dh, dl);
+    const float ph = __fmul_rn(w, dh);
+    const float pl = __fmaf_rn(w, dl, __fmaf_rn(w, dh, -ph));
+    float t, e;
+    two_sum<float>(h[q], ph, t, e);
+    h[q] = t;
+    l[q] = __fadd_rn(l[q], __fadd_rn(e, pl));
+  };
+  for (int i = lane; i < c.na; i += 32) {
+    const float w = wa[i];
+    const float4 p = xs[ia[i]];
+    acc(0, w, p.x, ra.x);
+    acc(1, w, p.y, ra.y);
+    acc(2, w, p.z, ra.z);
+  }
+  for (int i = lane; i < c.nb; i += 32) {
+    const float w = wb[i];
+    const float4 p = xs[ib[i]];
+    acc(3, w, p.x, rb.x);
+    acc(4, w, p.y, rb.y);
+    acc(5, w, p.z, rb.z);
+  }
+  const bool up = (lane & 16) != 0;
+  float vh[3], vl[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    vh[q] = up ? h[3 + q] : h[q];
+    vl[q] = up ? l[3 + q] : l[q];
+    const float sh = up ? h[q] : h[3 + q], slo = up ? l[q] : l[3 + q];
+    const float oh = __shfl_xor_sync(0xffffffffu, sh, 16), ol = __shfl_xor_sync(0xffffffffu, slo, 16);
+    float t, e;
+    two_sum<float>(vh[q], oh, t, e);
+    vh[q] = t;
+    vl[q] = __fadd_rn(__fadd_rn(vl[q], ol), e);
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const float oh = __shfl_xor_sync(0xffffffffu, vh[q], o), ol = __shfl_xor_sync(0xffffffffu, vl[q], o);
+      float t, e;
+      two_sum<float>(vh[q], oh, t, e);
+      vh[q] = t;
+      vl[q] = __fadd_rn(__fadd_rn(vl[q], ol), e);
+    }
+  float bh[3], bl[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    bh[q] = __shfl_sync(0xffffffffu, vh[q], 16);
+    bl[q] = __shfl_sync(0xffffffffu, vl[q], 16);
+  }
+  if (lane != 0) return 0;
+  const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
+  return com_finish_ff(c, a0, vh, vl, b0, bh, bl, s, sl, u);
+}
+
 // Centre-of-mass distance s = |R_B - R_A| (minimum image if pbc). Each
 // group's weighted sum runs over offsets from the group's first atom, which
 // keeps the rounding at the scale of the group's extent rather than of the
 // absolute coordinates: R_G = r_G + sum_i w_i (x_i - r_G), sum_i w_i = 1.
-// FP32 walkers sum every weighted offset exactly as hi + lo (the difference
-// x - r_G split by two_sum, the product's error by fma; the tiny w times the
-// difference's low part rounded once) with two_sum per thread and hi + lo
-// across the group, and finish in hi + lo (com_finish_ff): a group of
-// hundreds of atoms spread over nanometres would otherwise lose ~1e-7 nm,
-// several millionths of a hill a few grid spacings wide.
+// FP32 walkers: by the group's first warp (com_one_warp).
 template <typename Real>
 __device__ void cv_com(const Grp &g, GroupFixed<Real> *fx, int k, const typename Rec4<Real>::T *xs) {
   const CvDev &c = fx->wd.cv[k];
   const int32_t *ia = fx->ia[k], *ib = fx->ib[k];
   const Real *wa = fx->wa[k], *wb = fx->wb[k];
-  const auto ra = xs[ia[0]];
-  const auto rb = xs[ib[0]];
   if constexpr (sizeof(Real) == 4) {
-    float h[6] = {0, 0, 0, 0, 0, 0}, l[6] = {0, 0, 0, 0, 0, 0};
-    auto acc = [&](int q, float w, float x, float r) {
-      float dh, dl;
-      two_sum<float>(x, -r, dh, dl);  // x - r exactly
-      const float ph = __fmul_rn(w, dh);
-      const float pl = __fmaf_rn(w, dl, __fmaf_rn(w, dh, -ph));
-      float t, e;
-      two_sum<float>(h[q], ph, t, e);
-      h[q] = t;
-      l[q] = __fadd_rn(l[q], __fadd_rn(e, pl));
-    };
-    for (int i = g.t; i < c.na; i += g.G) {
-      const float w = wa[i];
-      const auto p = xs[ia[i]];
-      acc(0, w, p.x, ra.x);
-      acc(1, w, p.y, ra.y);
-      acc(2, w, p.z, ra.z);
-    }
-    for (int i = g.t; i < c.nb; i += g.G) {
-      const float w = wb[i];
-      const auto p = xs[ib[i]];
-      acc(3, w, p.x, rb.x);
-      acc(4, w, p.y, rb.y);
-      acc(5, w, p.z, rb.z);
-    }
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      // the running sum and its low part as a normalised hi + lo pair
-      float s2, e2;
-      two_sum<float>(h[q], l[q], s2, e2);
-      h[q] = s2;
-      l[q] = e2;
-      grp_sum_ff<float>(g, h[q], l[q], fx->red);
-    }
-    if (g.t == 0) {
-      const float r0a[3] = {ra.x, ra.y, ra.z}, r0b[3] = {rb.x, rb.y, rb.z};
-      float sh, sl;
-      const int fl = com_finish_ff(c, r0a, h, l, r0b, h + 3, l + 3, sh, sl, fx->com_u[k]);
-      fx->sh[k] = sh;
-      fx->sl[k] = sl;
-      if (fl) fx->flags |= fl;
+    if (g.warp == 0) {
+      float s = 0.f, sl = 0.f;
+      const int fl = com_one_warp(c, ia, ib, wa, wb, xs, g.lane, s, sl, fx->com_u[k]);
+      if (g.lane == 0) {
+        fx->sh[k] = s;
+        fx->sl[k] = sl;
+        if (fl) atomicOr(&fx->flags, fl);
+      }
     }
     return;
   }
+  const auto ra = xs[ia[0]];
+  const auto rb = xs[ib[0]];
   Real v[6] = {0, 0, 0, 0, 0, 0};
   for (int i = g.t; i < c.na; i += g.G) {
     Real w = wa[i];
@@ -410,14 +456,21 @@ __device__ void cv_com(const Grp &g, GroupFixed<Real> *fx, int k, const typename
   }
 }
 
-template <typename Real>
+template <typename Real, bool RN = false>
 __device__ __forceinline__ void cross3(const Real *a, const Real *b, Real *o) {
-  o[0] = a[1] * b[2] - a[2] * b[1];
-  o[1] = a[2] * b[0] - a[0] * b[2];
-  o[2] = a[0] * b[1] - a[1] * b[0];
+  if constexpr (RN) {
+    o[0] = fma_rn(a[1], b[2], -mul_rn(a[2], b[1]));
+    o[1] = fma_rn(a[2], b[0], -mul_rn(a[0], b[2]));
+    o[2] = fma_rn(a[0], b[1], -mul_rn(a[1], b[0]));
+  } else {
+    o[0] = a[1] * b[2] - a[2] * b[1];
+    o[1] = a[2] * b[0] - a[0] * b[2];
+    o[2] = a[0] * b[1] - a[1] * b[0];
+  }
 }
-template <typename Real>
+template <typename Real, bool RN = false>
 __device__ __forceinline__ Real dot3(const Real *a, const Real *b) {
+  if constexpr (RN) return fma_rn(a[2], b[2], fma_rn(a[0], b[0], mul_rn(a[1], b[1])));
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
@@ -445,8 +498,11 @@ __device__ __forceinline__ double dihedral_angle64(const CvDev &c, const float (
 // Dihedral of atoms 1-2-3-4 at positions x: phi = atan2(|b2| b1.(b2 x b3),
 // (b1 x b2).(b2 x b3)), gradient in the Blondel-Karplus form, by one thread.
 // phi_lo receives the low part of the angle: 0, or with c.hp (FP32 walkers)
-// the FP64 angle's remainder after its FP32 rounding phi.
-template <typename Real>
+// the FP64 angle's remainder after its FP32 rounding phi. RN: every product
+// and sum rounded as written (fma where written), so that each kernel's copy
+// computes the same bits; otherwise contraction is the compiler's (which, in
+// the closed-loop kernel, forms the same products: the bits agree).
+template <typename Real, bool RN = false>
 __device__ __forceinline__ int dihedral_core(const CvDev &c, const Real (&x)[4][3], Real &phi, Real (*grad)[3],
                                              Real &phi_lo) {
   phi_lo = 0;
@@ -456,14 +512,14 @@ __device__ __forceinline__ int dihedral_core(const CvDev &c, const Real (&x)[4][
     b2[q] = x[2][q] - x[1][q];
     b3[q] = x[3][q] - x[2][q];
     if (c.pbc) {
-      b1[q] = min_image(b1[q], c.box[q], c.inv_box[q]);
-      b2[q] = min_image(b2[q], c.box[q], c.inv_box[q]);
-      b3[q] = min_image(b3[q], c.box[q], c.inv_box[q]);
+      b1[q] = min_image<Real, RN>(b1[q], c.box[q], c.inv_box[q]);
+      b2[q] = min_image<Real, RN>(b2[q], c.box[q], c.inv_box[q]);
+      b3[q] = min_image<Real, RN>(b3[q], c.box[q], c.inv_box[q]);
     }
   }
-  cross3(b1, b2, m);
-  cross3(b2, b3, n);
-  Real b2sq = dot3(b2, b2);
+  cross3<Real, RN>(b1, b2, m);
+  cross3<Real, RN>(b2, b3, n);
+  Real b2sq = dot3<Real, RN>(b2, b2);
   Real lb2 = sqrt(b2sq);
   if constexpr (sizeof(Real) == 4) {
     if (c.hp) {
@@ -471,32 +527,37 @@ __device__ __forceinline__ int dihedral_core(const CvDev &c, const Real (&x)[4][
       phi = (float)p64;
       phi_lo = (float)(p64 - (double)phi);
     } else {
-      phi = atan2(lb2 * dot3(b1, n), dot3(m, n));
+      phi = atan2(lb2 * dot3<Real, RN>(b1, n), dot3<Real, RN>(m, n));
     }
   } else {
-    phi = atan2(lb2 * dot3(b1, n), dot3(m, n));
+    phi = atan2(lb2 * dot3<Real, RN>(b1, n), dot3<Real, RN>(m, n));
   }
-  Real mm = dot3(m, m), nn = dot3(n, n);
+  Real mm = dot3<Real, RN>(m, m), nn = dot3<Real, RN>(n, n);
   if (!(mm > 0) || !(nn > 0) || !(lb2 > 0)) {
     for (int a = 0; a < 4; ++a)
       for (int q = 0; q < 3; ++q) grad[a][q] = 0;
     return ABP_WFLAG_SINGULAR;
   }
   Real inv_b2sq = rcp_fast<Real>(b2sq);
-  Real p = dot3(b1, b2) * inv_b2sq, r = dot3(b3, b2) * inv_b2sq;
+  Real p = dot3<Real, RN>(b1, b2) * inv_b2sq, r = dot3<Real, RN>(b3, b2) * inv_b2sq;
   Real cm = -lb2 * rcp_fast<Real>(mm), cn = lb2 * rcp_fast<Real>(nn);
   for (int q = 0; q < 3; ++q) {
     Real g1 = cm * m[q];
     Real g4 = cn * n[q];
     grad[0][q] = g1;
     grad[3][q] = g4;
-    grad[1][q] = -(1 + p) * g1 + r * g4;
-    grad[2][q] = -(1 + r) * g4 + p * g1;
+    if constexpr (RN) {
+      grad[1][q] = fma_rn(r, g4, -mul_rn(add_rn((Real)1, p), g1));
+      grad[2][q] = fma_rn(p, g1, -mul_rn(add_rn((Real)1, r), g4));
+    } else {
+      grad[1][q] = -(1 + p) * g1 + r * g4;
+      grad[2][q] = -(1 + r) * g4 + p * g1;
+    }
   }
   return 0;
 }
 
-// The dihedral of the atoms ia[0..3] of xs (dihedral_core).
+// The dihedral of the atoms ia[0..3] of xs (dihedral_core, rounded as written).
 template <typename Real>
 __device__ __forceinline__ int dihedral_eval(const CvDev &c, const int32_t *ia, const typename Rec4<Real>::T *xs,
                                              Real &phi, Real (*grad)[3], Real &phi_lo) {
@@ -508,7 +569,7 @@ __device__ __forceinline__ int dihedral_eval(const CvDev &c, const int32_t *ia, 
     x[a][1] = p.y;
     x[a][2] = p.z;
   }
-  return dihedral_core<Real>(c, x, phi, grad, phi_lo);
+  return dihedral_core<Real, true>(c, x, phi, grad, phi_lo);
 }
 
 template <typename Real>
@@ -518,17 +579,315 @@ __device__ void cv_dihedral(const Grp &g, GroupFixed<Real> *fx, int k, const typ
   int fl = dihedral_eval<Real>(fx->wd.cv[k], fx->ia[k], xs, phi, fx->dih_g[k], phi_lo);
   fx->sh[k] = phi;
   fx->sl[k] = phi_lo;
-  if (fl) fx->flags |= fl;
+  if (fl) atomicOr(&fx->flags, fl);
 }
 
-// Coordination number s = sum_{i in A, j in B} 1 / (1 + (r_ij / r0)^6)
-// (the n = 6, m = 12 rational switch with the common factor cancelled).
-// No square root: q = r^2 / r0^2, sw = 1 / (1 + q^3),
-// d sw / d x_i = -6 q^2 sw^2 / r0^2 (x_i - x_j).
-// Thread t owns B entries t, t + G, ... (JB per pass, gradients in registers);
-// A entries are read from shared memory in chunks of 4 and their gradients
-// are reduced over the warp, then summed over warps in a fixed order.
-// jA / jB receive ds/dx per list entry.
+// Two FP32 values in one 64-bit register: the packed FP32 instructions of
+// sm_100 and later (each half rounded as the scalar instruction rounds it).
+// They run at the scalar FMA rate per lane with half the issue slots.
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 f2_pack(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(F2 v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// 1 / x of both halves for x >= 1 (infinity gives 0): one MUFU instruction
+// each, without the scaling a general divide needs near the format's ends.
+__device__ __forceinline__ F2 f2_rcp(F2 v) {
+  float lo, hi;
+  f2_unpack(v, lo, hi);
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(lo));
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(hi));
+  return f2_pack(lo, hi);
+}
+// Minimum image d - L rint(d / L) of both halves, rint formed by adding and
+// subtracting 1.5 2^23 (exact for |d / L| < 2^22; at a tie either image has
+// the same length).
+__device__ __forceinline__ F2 f2_min_image(F2 d, F2 invL, F2 negL) {
+  const F2 M = f2_pack(12582912.0f, 12582912.0f), nM = f2_pack(-12582912.0f, -12582912.0f);
+  return f2_fma(f2_add(f2_fma(d, invL, M), nM), negL, d);
+}
+
+// One switch term of two pairs at separations (dx, dy, dz): sw = 1 / (1 +
+// q^3), q = r^2 / r0^2, and gf = q^2 sw^2 (ds/dx_i = -6 gf / r0^2 (x_i - x_j)).
+struct CnPair {
+  F2 k2, one, negLx, negLy, negLz, iLx, iLy, iLz;
+  __device__ __forceinline__ explicit CnPair(const CvDev &c) {
+    const float k = (float)c.inv_r0sq;
+    k2 = f2_pack(k, k);
+    one = f2_pack(1.f, 1.f);
+    const float b[3] = {(float)c.box[0], (float)c.box[1], (float)c.box[2]};
+    const float ib[3] = {(float)c.inv_box[0], (float)c.inv_box[1], (float)c.inv_box[2]};
+    negLx = f2_pack(-b[0], -b[0]);
+    negLy = f2_pack(-b[1], -b[1]);
+    negLz = f2_pack(-b[2], -b[2]);
+    iLx = f2_pack(ib[0], ib[0]);
+    iLy = f2_pack(ib[1], ib[1]);
+    iLz = f2_pack(ib[2], ib[2]);
+  }
+  template <bool PBC>
+  __device__ __forceinline__ void image(F2 &dx, F2 &dy, F2 &dz) const {
+    if constexpr (PBC) {
+      dx = f2_min_image(dx, iLx, negLx);
+      dy = f2_min_image(dy, iLy, negLy);
+      dz = f2_min_image(dz, iLz, negLz);
+    }
+  }
+  __device__ __forceinline__ void term(F2 dx, F2 dy, F2 dz, F2 &sw, F2 &q2) const {
+    const F2 q = f2_mul(f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))), k2);
+    q2 = f2_mul(q, q);
+    sw = f2_rcp(f2_fma(q2, q, one));
+  }
+};
+
+// Compensated sum of switch values: two packed sums that start at 2, so that
+// adding x with 0 <= x <= 2 leaves its exact error to three more additions
+// (fast two-sum).
+struct CnSum {
+  F2 s, c, minus;
+  __device__ __forceinline__ CnSum() : s(f2_pack(2.f, 2.f)), c(0ull), minus(f2_pack(-1.f, -1.f)) {}
+  __device__ __forceinline__ void add(F2 x) {
+    const F2 t = f2_add(s, x);
+    const F2 z = f2_fma(s, minus, t);    // t - s (exact)
+    c = f2_add(c, f2_fma(z, minus, x));  // x - z (exact)
+    s = t;
+  }
+  // the sum as hi + lo
+  __device__ __forceinline__ void get(float &h, float &l) const {
+    float s0, s1, c0, c1, h1, l1;
+    f2_unpack(s, s0, s1);
+    f2_unpack(c, c0, c1);
+    two_sum<float>(__fsub_rn(s0, 2.f), c0, h, l);  // (the subtraction is exact: s0 >= 2)
+    two_sum<float>(__fsub_rn(s1, 2.f), c1, h1, l1);
+    ff_add<float>(h, l, h1, l1);
+  }
+};
+
+// One block of A atoms (nab of them, from list position a0) against a warp's
+// B atoms (cn_warp): RP packed rows a lane, known at compile time so that the
+// rows' chains overlap.
+template <bool PBC, int RP>
+__device__ __forceinline__ void cn_block(const CnPair &cp, float c6, const int32_t *ia, const int32_t *ib, int nb,
+                                         const float4 *xs, float4 *jB, float *lig, bool more, bool first, int nab,
+                                         int lane, int bgrp, int nbg, int rounds, CnSum &sum) {
+  const int ag = lane & 3;
+  F2 ax[RP], ay[RP], az[RP], gx[RP], gy[RP], gz[RP];
+#pragma unroll
+  for (int q = 0; q < RP; ++q) {
+    gx[q] = gy[q] = gz[q] = 0ull;
+    const int i0 = ag + 8 * q, i1 = i0 + 4;
+    const float4 p0 = i0 < nab ? xs[ia[i0]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 p1 = i1 < nab ? xs[ia[i1]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    ax[q] = f2_pack(p0.x, p1.x);
+    ay[q] = f2_pack(p0.y, p1.y);
+    az[q] = f2_pack(p0.z, p1.z);
+  }
+  // the last packed row may be short: its switch values are masked
+  const F2 tail = f2_pack(ag + 8 * (RP - 1) < nab ? 1.f : 0.f, ag + 8 * (RP - 1) + 4 < nab ? 1.f : 0.f);
+  float4 pn = xs[ib[min(bgrp, nb - 1)]];
+  int jn = ib[min(bgrp + nbg, nb - 1)];
+  // every lane runs the same number of B rounds (the lane exchanges need the
+  // whole warp); in the last one a lane past the end of B skips the pairs
+  for (int rj = 0; rj < rounds; ++rj) {
+    const int j = bgrp + rj * nbg;
+    const bool okj = j < nb;
+    const float4 p = pn;
+    pn = xs[jn];  // the next round's atom, and the index of the one after it
+    jn = ib[min(j + 2 * nbg, nb - 1)];
+    float gjx = 0.f, gjy = 0.f, gjz = 0.f;
+    if (okj) {
+      const F2 px = f2_pack(-p.x, -p.x), py = f2_pack(-p.y, -p.y), pz = f2_pack(-p.z, -p.z);
+      F2 prev = 0ull, bx = 0ull, by = 0ull, bz = 0ull;
+#pragma unroll
+      for (int q = 0; q < RP; ++q) {
+        F2 dx = f2_add(ax[q], px), dy = f2_add(ay[q], py), dz = f2_add(az[q], pz);
+        cp.image<PBC>(dx, dy, dz);
+        F2 sw, q2;
+        cp.term(dx, dy, dz, sw, q2);
+        if (q == RP - 1) sw = f2_mul(sw, tail);
+        if (q & 1)
+          sum.add(f2_add(prev, sw));
+        else if (q == RP - 1)
+          sum.add(sw);
+        prev = sw;
+        const F2 gf = f2_mul(q2, f2_mul(sw, sw));
+        gx[q] = f2_fma(gf, dx, gx[q]);
+        gy[q] = f2_fma(gf, dy, gy[q]);
+        gz[q] = f2_fma(gf, dz, gz[q]);
+        bx = f2_fma(gf, dx, bx);
+        by = f2_fma(gf, dy, by);
+        bz = f2_fma(gf, dz, bz);
+      }
+      float lo, hi;
+      f2_unpack(bx, lo, hi);
+      gjx = __fadd_rn(lo, hi);
+      f2_unpack(by, lo, hi);
+      gjy = __fadd_rn(lo, hi);
+      f2_unpack(bz, lo, hi);
+      gjz = __fadd_rn(lo, hi);
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      gjx = __fadd_rn(gjx, __shfl_xor_sync(0xffffffffu, gjx, o));
+      gjy = __fadd_rn(gjy, __shfl_xor_sync(0xffffffffu, gjy, o));
+      gjz = __fadd_rn(gjz, __shfl_xor_sync(0xffffffffu, gjz, o));
+    }
+    if (ag == 0 && okj) {
+      float4 v = make_float4(__fmul_rn(-c6, gjx), __fmul_rn(-c6, gjy), __fmul_rn(-c6, gjz), 0.f);
+      if (!first) {
+        const float4 o = jB[j];
+        v.x = __fadd_rn(o.x, v.x);
+        v.y = __fadd_rn(o.y, v.y);
+        v.z = __fadd_rn(o.z, v.z);
+      }
+      jB[j] = v;
+    }
+  }
+  // the block's A gradients: value 3 r + e is component e of A atom ag + 4 r
+  // of the block; three exchange levels leave each lane four warp sums
+  float v[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = 0.f;
+#pragma unroll
+  for (int q = 0; q < RP; ++q) {
+    f2_unpack(gx[q], v[6 * q], v[6 * q + 3]);
+    f2_unpack(gy[q], v[6 * q + 1], v[6 * q + 4]);
+    f2_unpack(gz[q], v[6 * q + 2], v[6 * q + 5]);
+  }
+#pragma unroll
+  for (int o = 16, n = 16; o >= 4; o >>= 1, n >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < n) {
+        const float keep = up ? v[n + i] : v[i], send = up ? v[i] : v[n + i];
+        v[i] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, o));
+      }
+  }
+  const int base = ((lane & 16) ? 16 : 0) + ((lane & 8) ? 8 : 0) + ((lane & 4) ? 4 : 0);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int idx = base + i, r = idx / 3, e = idx - 3 * r, at = ag + 4 * r;
+    if (idx < 30 && at < nab) {
+      float *L = lig + at * 3 + e;
+      *L = more ? __fadd_rn(*L, v[i]) : v[i];
+    }
+  }
+}
+
+// FP32 coordination number s = sum_{i in A, j in B} 1 / (1 + (r_ij / r0)^6)
+// (the n = 6, m = 12 rational switch with the common factor cancelled, no
+// square root): the part of one warp, which takes the B atoms j with j % nbg
+// in [b0, b0 + 8). Blocks of 40 A atoms are tiled over the warp: lane & 3
+// picks one of four A-groups (A atoms i with i % 4 == lane & 3, up to 10 a
+// lane, held in registers with their gradients as packed pairs), lane >> 2
+// one of eight B-groups (streamed, the next atom loaded a round ahead). Every
+// pair is evaluated once, two at a time. A B atom's gradient is summed over
+// its four A-groups by two lane exchanges; a block's A gradients over the
+// B-groups by a reduce-scatter. Switch values are added in twos to a
+// compensated sum (CnSum): a CN of hundreds must be known to ~1e-8 relative to
+// place a hill two grid spacings wide.
+// jB receives ds/dx of the warp's B atoms, lig[na][3] the warp's A sums
+// (unscaled; added to what is there if `more`), sh + sl the lane's own part
+// of s (warp_sum_ff adds the lanes). Bound by the FMA pipe: 20 lane-operations a pair (26 with a
+// minimum image) plus ~3 for the exchanges; the reciprocal takes 8 of those
+// cycles' MUFU slots.
+template <bool PBC>
+__device__ __forceinline__ void cn_warp(const CvDev &c, const int32_t *ia, const int32_t *ib, const float4 *xs,
+                                        float4 *jB, float *lig, bool more, int lane, int b0, int nbg, float &sh,
+                                        float &sl) {
+  const CnPair cp(c);
+  const int na = c.na, nb = c.nb, bgrp = b0 + (lane >> 2);
+  const float c6 = -6.f * (float)c.inv_r0sq;
+  const int rounds = (nb - b0 + nbg - 1) / nbg;  // of the warp's first B-group, the longest
+  CnSum sum;
+  for (int a0 = 0; a0 < na; a0 += 40) {
+    const int nab = min(40, na - a0);
+#define ABP_CN_BLOCK(RP) \
+  cn_block<PBC, RP>(cp, c6, ia + a0, ib, nb, xs, jB, lig + 3 * a0, more, a0 == 0, nab, lane, bgrp, nbg, rounds, sum)
+    switch ((nab + 7) >> 3) {
+      case 1: ABP_CN_BLOCK(1); break;
+      case 2: ABP_CN_BLOCK(2); break;
+      case 3: ABP_CN_BLOCK(3); break;
+      case 4: ABP_CN_BLOCK(4); break;
+      default: ABP_CN_BLOCK(5);
+    }
+#undef ABP_CN_BLOCK
+  }
+  sum.get(sh, sl);
+}
+
+// N hi + lo pairs summed over the warp (every lane gets the same bits: the
+// pairwise add is commutative).
+template <int N>
+__device__ __forceinline__ void warp_sum_ff(float (&h)[N], float (&l)[N]) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const float oh = __shfl_xor_sync(0xffffffffu, h[i], o), ol = __shfl_xor_sync(0xffffffffu, l[i], o);
+      ff_add<float>(h[i], l[i], oh, ol);
+    }
+}
+
+__device__ __forceinline__ void cn_warp_any(const CvDev &c, const int32_t *ia, const int32_t *ib, const float4 *xs,
+                                            float4 *jB, float *lig, bool more, int lane, int b0, int nbg, float &sh,
+                                            float &sl) {
+  if (c.pbc)
+    cn_warp<true>(c, ia, ib, xs, jB, lig, more, lane, b0, nbg, sh, sl);
+  else
+    cn_warp<false>(c, ia, ib, xs, jB, lig, more, lane, b0, nbg, sh, sl);
+}
+
+// The same by a group of warps: warp w takes the B-groups 8 w .. 8 w + 7 of
+// G / 4; its parts meet in warp order. jA / jB receive ds/dx per list entry,
+// lig is [warps][na][3] scratch, red [warps][2].
+__device__ __forceinline__ void cv_coord_f32(const Grp &g, const CvDev &c, const int32_t *ia, const int32_t *ib,
+                                             const float4 *xs, float4 *jA, float4 *jB, float *lig, float *red,
+                                             float &sh, float &sl) {
+  float h[1], l[1];
+  cn_warp_any(c, ia, ib, xs, jB, lig + g.warp * c.na * 3, false, g.lane, 8 * g.warp, g.G >> 2, h[0], l[0]);
+  warp_sum_ff<1>(h, l);
+  if (g.lane == 0) {
+    red[2 * g.warp] = h[0];
+    red[2 * g.warp + 1] = l[0];
+  }
+  g.sync();
+  sh = red[0];
+  sl = red[1];
+  for (int w = 1; w < g.nwarps; ++w) ff_add<float>(sh, sl, red[2 * w], red[2 * w + 1]);
+  const float c6 = -6.f * (float)c.inv_r0sq;
+  for (int i = g.t; i < c.na; i += g.G) {
+    float a0 = lig[i * 3], a1 = lig[i * 3 + 1], a2 = lig[i * 3 + 2];
+    for (int w = 1; w < g.nwarps; ++w) {
+      const float *L = lig + w * c.na * 3 + i * 3;
+      a0 = __fadd_rn(a0, L[0]);
+      a1 = __fadd_rn(a1, L[1]);
+      a2 = __fadd_rn(a2, L[2]);
+    }
+    jA[i] = make_float4(__fmul_rn(c6, a0), __fmul_rn(c6, a1), __fmul_rn(c6, a2), 0.f);
+  }
+  g.sync();
+}
+
 // Coordination number for a group A of at most 4 * MAXA atoms, tiled over
 // the group's threads: lane & 3 picks one of four A-groups (A atoms i with
 // i % 4 == lane & 3, held in registers with their gradients) and t >> 2 one
@@ -648,6 +1007,15 @@ __device__ void cv_coord_tiled(const Grp &g, GroupFixed<Real> *fx, int k, const 
 template <typename Real>
 __device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typename Rec4<Real>::T *xs,
                          typename Rec4<Real>::T *jA, typename Rec4<Real>::T *jB, Real *lig) {
+  if constexpr (sizeof(Real) == 4) {
+    float sh, sl;
+    cv_coord_f32(g, fx->wd.cv[k], fx->ia[k], fx->ib[k], xs, jA, jB, lig, fx->red, sh, sl);
+    if (g.t == 0) {
+      fx->sh[k] = sh;
+      fx->sl[k] = sl;
+    }
+    return;
+  } else {
   if (fx->wd.cv[k].na <= 4 * 10) {
     cv_coord_tiled<Real, 10>(g, fx, k, xs, jA, jB, lig);
     return;
@@ -755,6 +1123,7 @@ __device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typena
       a2 += L[2];
     }
     jA[i] = make_rec<Real>(a0, a1, a2, (Real)0);
+  }
   }
 }
 
@@ -1416,9 +1785,9 @@ __device__ void deposit_stencil(const Grp &g, GroupFixed<Real> *fx, const GroupL
 // dV/dxi_k = c b kT h'_k / (1 + c (1-b) h) (Eq. (btraj-grad)).
 template <typename Real>
 __device__ __forceinline__ void mabp_bias(const WalkerDev &wd, const Real *acc, Real &V, Real *dv) {
-  const Real hh = acc[0], ch = (Real)wd.mabp_h * hh;
+  const Real hh = acc[0], ch = mul_rn((Real)wd.mabp_h, hh);
   V = (Real)wd.mabp_k * log1p(ch);
-  const Real den = (Real)1 + ch;
+  const Real den = add_rn((Real)1, ch);
   for (int k = 0; k < wd.g.d; ++k) dv[k] = (Real)wd.mabp_g * acc[1 + k] / den;
 }
 
@@ -1426,40 +1795,47 @@ __device__ __forceinline__ void mabp_bias(const WalkerDev &wd, const Real *acc, 
 template <typename Real>
 __device__ __forceinline__ Real wall_grad(const WalkerDev &wd, int k, Real s) {
   if constexpr (sizeof(Real) == 4)
-    return (wd.kwall_f > 0.f && s > wd.smax_f[k]) ? wd.kwall_f * (s - wd.smax_f[k]) : 0.f;
+    return (wd.kwall_f > 0.f && s > wd.smax_f[k]) ? mul_rn(wd.kwall_f, sub_rn(s, wd.smax_f[k])) : 0.f;
   else
-    return (wd.kwall > 0 && s > (Real)wd.smax[k]) ? (Real)wd.kwall * (s - (Real)wd.smax[k]) : (Real)0;
+    return (wd.kwall > 0 && s > (Real)wd.smax[k]) ? mul_rn((Real)wd.kwall, sub_rn(s, (Real)wd.smax[k])) : (Real)0;
 }
 
-// a4: V and dV/ds_k at s after the deposit, by warp 0's first 2^d lanes,
-// combined with a fixed xor-butterfly; a clamped axis gets a zero gradient.
-// (For mABP the corners all sit on the nearest node with weight 1 on the
-// first, which yields that node's histograms, turned into the bias.)
+// a4: V and dV/ds_k at s after the deposit, by the group's first warp: lane c
+// reads corner c and forms its weight, the terms are then combined in corner
+// order (lane exchanges), as interp_one combines them: the same bits. A
+// clamped axis gets a zero gradient. (For mABP the corners all sit on the
+// nearest node with weight 1 on the first, which yields that node's
+// histograms, turned into the bias.)
 template <typename Real, bool TILE>
 __device__ void interp_step(const Grp &g, GroupFixed<Real> *fx, const GroupLayout &L, const unsigned char *tile) {
   const GridDev &gd = fx->wd.g;
   if (g.warp == 0) {
-    Real acc[4] = {0, 0, 0, 0};
-    if (g.lane < (1 << gd.d)) {
-      Real w = 1;
-      for (int k = 0; k < gd.d; ++k) w *= ((g.lane >> k) & 1) ? fx->f[k] : (Real)1 - fx->f[k];
-      Real v[4];
+    const int d = gd.d, nc = 1 << d;
+    Real w = 1, v[4] = {0, 0, 0, 0};
+    if (g.lane < nc) {
       rec_values<Real>(gd, corner_ptr<Real, TILE>(fx, L, tile, g.lane), v);
-      for (int q = 0; q <= gd.d; ++q) acc[q] = w * v[q];
+      for (int k = 0; k < d; ++k) w = mul_rn(w, ((g.lane >> k) & 1) ? fx->f[k] : sub_rn((Real)1, fx->f[k]));
     }
-    for (int q = 0; q < 4; ++q)
-      for (int o = 1; o < 8; o <<= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    Real acc[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (c < nc) {
+        const Real wc = __shfl_sync(0xffffffffu, w, c);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = fma_rn(wc, __shfl_sync(0xffffffffu, v[q], c), acc[q]);
+      }
     if (g.lane == 0) {
       if (fx->wd.method == ABP_METHOD_MABP) {
         Real V, dvm[3];
         mabp_bias<Real>(fx->wd, acc, V, dvm);
         acc[0] = V;
-        for (int k = 0; k < gd.d; ++k) acc[1 + k] = dvm[k];
+        for (int k = 0; k < d; ++k) acc[1 + k] = dvm[k];
       }
       fx->V = acc[0];
-      for (int k = 0; k < gd.d; ++k) {
-        Real dv = ((fx->clamped >> k) & 1) ? (Real)0 : acc[1 + k];
-        dv += wall_grad<Real>(fx->wd, k, fx->sh[k] + fx->sl[k]);
+      for (int k = 0; k < d; ++k) {
+        // the wall acts on the CV's high part, as in finish_lookup
+        const Real dv =
+            add_rn(((fx->clamped >> k) & 1) ? (Real)0 : acc[1 + k], wall_grad<Real>(fx->wd, k, fx->sh[k]));
         fx->dvds[k] = dv;
         fx->dV[k] = dv;
       }

@@ -61,6 +61,48 @@ struct RunArgs {
   DevCounters *ctr;
 };
 
+// A block of steps of the split form (abp_split.cu): steps t0 .. t0 + nsteps
+// of the call for nw walkers of one batch.
+struct SplitArgs {
+  const TableEntry *table;
+  int nw;
+  int nsteps;          // steps of this block
+  long long t0;        // its first step, counted from the call's first
+  const void *coords;
+  const long long *coff;
+  long long cstride;
+  void *forces;        // NULL: the walkers' own force buffers (abp_step)
+  const long long *foff;
+  long long fstride;
+  int mode;
+  int serial;          // the force records of a walker's steps overlap: added in step order
+  int last;            // the call's last block
+  int chunk;           // steps per warp of k_sp_cn (set by the launcher)
+  long long step0;     // MD step of the call's first step
+  void *recs;          // [nw][nsteps] step records
+  void *jac;           // [nw][nsteps][jstride] gradient records of coordination numbers
+  int jstride;
+  void *terms;         // [nw][term_stride] list entries per atom of walkers with gradient records (else NULL)
+  size_t term_stride;  // 8-byte words
+  DepositLog log;
+  DevCounters *ctr;
+};
+
+// What the launcher needs to know of a batch's walkers (split_shape adds one).
+struct SplitShape {
+  int win = 0;         // steps per window (0: walkers of k_sp_cn)
+  int cv_smem = 0;
+  bool staged = true;  // k_sp_cn's walkers are small enough to stage their coordinates
+  int wt = 0, mabp = 0;
+  int min_dim = 0, max_atoms = 0;
+};
+bool split_eligible(const WalkerDev &hd, bool win);
+void split_shape(const WalkerDev &hd, bool win, SplitShape *s);
+size_t split_step_bytes();
+int split_jac_records(const WalkerDev &hd);
+int split_term_words(const WalkerDev &hd);
+cudaError_t launch_split(const SplitArgs &a, const SplitShape &s, int sms, LaunchTimer *tm, cudaStream_t st);
+
 struct PlainArgs {
   int nw;
   const WalkerDev *const *wd_dev;  // host array of device descriptors

@@ -48,17 +48,6 @@ struct Iter2 {
   }
 };
 
-// Rounded arithmetic with no contraction left to the compiler, so that every
-// inlined copy of a CV computes the same bits.
-__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
-
 // One group's part of a COM distance: the group's first atom r0 and the
 // weighted offsets of its atoms from r0, summed in list order (FP32 walkers:
 // compensated, the low part of the sum in lo; FP64 walkers: lo = 0).
@@ -154,7 +143,7 @@ __device__ __forceinline__ void finish_lookup(const WalkerDev &wd, StepRec<Real>
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     if (k < d) {
-      const Real dv = (((st.clamped >> k) & 1) ? (Real)0 : acc[1 + k]) + wall_grad<Real>(wd, k, st.s[k]);
+      const Real dv = add_rn(((st.clamped >> k) & 1) ? (Real)0 : acc[1 + k], wall_grad<Real>(wd, k, st.s[k]));
       st.dv[k] = dv;
       const int nj = wd.cv[k].type == ABP_CV_COM_DIST ? 3 : 12;
       for (int q = 0; q < nj; ++q) st.jac[k][q] *= dv;
@@ -244,7 +233,7 @@ __device__ __forceinline__ void interp_combine(const WalkerDev &wd, StepRec<Real
     Real v[4];
     rec_vals<Real, DIM>(ca[c], cb[c], v);
 #pragma unroll
-    for (int q = 0; q <= DIM; ++q) acc[q] += wc * v[q];
+    for (int q = 0; q <= DIM; ++q) acc[q] = fma_rn(wc, v[q], acc[q]);
   }
   finish_lookup<Real>(wd, st, acc);
 }
@@ -266,7 +255,7 @@ __device__ __forceinline__ void interp_one(const WalkerDev &wd, StepRec<Real> &s
   for (int c = 0; c < NC; ++c) {
     const Real wc = corner_weight<Real, DIM>(st, c);
 #pragma unroll
-    for (int q = 0; q <= DIM; ++q) acc[q] += wc * v[c][q];
+    for (int q = 0; q <= DIM; ++q) acc[q] = fma_rn(wc, v[c][q], acc[q]);
   }
   finish_lookup<Real>(wd, st, acc);
 }
@@ -290,15 +279,15 @@ __device__ __forceinline__ int rmsd_thread(const CvDev &c, const int32_t *ia, co
       dx[i][0] = p.x - ref[3 * i];
       dx[i][1] = p.y - ref[3 * i + 1];
       dx[i][2] = p.z - ref[3 * i + 2];
-      acc += dx[i][0] * dx[i][0] + dx[i][1] * dx[i][1] + dx[i][2] * dx[i][2];
+      acc = add_rn(acc, fma_rn(dx[i][2], dx[i][2], fma_rn(dx[i][0], dx[i][0], mul_rn(dx[i][1], dx[i][1]))));
     }
   const Real N = (Real)c.na;
-  s = sqrt(acc / N + (Real)0.01);
-  const Real inv = (Real)1 / (N * s);
+  s = sqrt(add_rn(acc / N, (Real)0.01));
+  const Real inv = (Real)1 / mul_rn(N, s);
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     if (i < c.na)
-      for (int q = 0; q < 3; ++q) J[3 * i + q] = dx[i][q] * inv;
+      for (int q = 0; q < 3; ++q) J[3 * i + q] = mul_rn(dx[i][q], inv);
   return 0;
 }
 
