@@ -680,6 +680,8 @@ abp_status upload(abp_walker *w, const void *src, size_t bytes, void **dst) {
 void walker_free(abp_walker *w) {
   for (auto &a : w->allocs) dev_free(w->ctx, a.first, a.second);
   w->allocs.clear();
+  if (w->hd.bpart) cudaFree(w->hd.bpart);
+  w->hd.bpart = nullptr;
 }
 
 abp_status check_indices(const int32_t *idx, int n, int natoms, const char *what, int k) {
@@ -984,6 +986,15 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
   }
   if (st == ABP_OK && w->big && big_cn_smem(hd) > 200 * 1024)
     st = fail(ABP_ERR_UNSUPPORTED, "a coordination number with more than ~2000 A atoms is not built");
+  if (st == ABP_OK && w->big && big_part_bytes(hd) > 0) {
+    // (not counted against the budget, which is for grids and walkers)
+    if (cudaMalloc(&p, big_part_bytes(hd)) != cudaSuccess) {
+      cudaGetLastError();
+      st = fail(ABP_ERR_OOM, "cudaMalloc of %zu bytes for partial sums", big_part_bytes(hd));
+    } else {
+      hd.bpart = p;
+    }
+  }
   if (st == ABP_OK && w->big) {
     // the force phase's per-atom term table, into the walker's scratch
     std::vector<int32_t> terms;
@@ -1073,6 +1084,12 @@ static abp_status sub_table(abp_ctx *ctx, const std::vector<abp_walker *> &ws, c
   victim->last_use = ctx->use_clock;
   *out = victim->dev;
   return ABP_OK;
+}
+
+static bool any_deposit(const std::vector<abp_walker *> &ws, long long step) {
+  for (const abp_walker *w : ws)
+    if (step % w->hd.stride == 0) return true;
+  return false;
 }
 
 // Items of the phased form: one per walker, then one per CN chunk.
@@ -1288,6 +1305,7 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     b.timer = ctx->timer;
     for (int t = 0; t < nsteps; ++t) {
       b.step = step0 + t;
+      b.any_deposit = any_deposit(bw, b.step);
       b.step_off = (long long)t * cstride;
       b.force_step_off = (long long)t * fstride;
       cudaError_t e = launch_big_step(b, ctx->stream);
@@ -1446,6 +1464,7 @@ abp_status abp_md_run(abp_ctx *ctx, abp_walker *const *walkers, int n, void *coo
     b.toff = reinterpret_cast<const long long *>(traj_offsets_dev);
     for (int t = 0; t < nsteps; ++t) {
       b.step = step0 + t;
+      b.any_deposit = any_deposit(bw, b.step);
       b.step_off = 0;  // the coordinates stay where they are and move in place
       b.force_step_off = (long long)t * force_step_stride;
       b.traj_step_off = (long long)t * traj_step_stride;

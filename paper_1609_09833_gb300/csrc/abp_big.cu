@@ -1,19 +1,28 @@
 // abp_big.cu -- the phased form of the force call, for walkers that share a
 // grid (multiple-walker runs) or that are too large for one shared-memory
-// walker group. One MD step is five launches over all such walkers:
+// walker group. One MD step is three launches over all such walkers, six on a
+// step that deposits:
 //
 //   k_big_cn       a1, coordination numbers: the A x B pair sum split over
 //                  CTAs by chunks of B (kBigChunk entries); each CTA writes
-//                  dCN/dx of its B entries and its partial CN and A gradients
+//                  dCN/dx of its B entries, its partial CN and A gradients,
+//                  and whether its share of the walker's atoms is finite
 //   k_big_cvs      a1 (other CVs, partial sums combined in chunk order) and
 //                  a2: every walker's hill height from the grid as it was
-//                  before any deposit of the step (Jacobi order)
+//                  before any deposit of the step (Jacobi order); on a step
+//                  without deposits a4 as well
 //   k_big_deposit  a3: the hills; shared grids add them to the FP64 shadow
 //                  with atomics (order-independent up to FP64 rounding), own
 //                  grids with the two-sum update of the fused form
 //   k_big_refresh  shared grids: FP32 fields = FP64 shadow split into
 //                  value + compensation (about 48 bits kept)
-//   k_big_force    a4 + a5: interpolation after all deposits, chain rule
+//   k_big_lookup   a4 after all deposits
+//   k_big_force    a5, and in a closed loop the move of the atoms
+//
+// Each may start while the one before it ends (launch_chained). 32 walkers on a
+// shared 256^3 grid, 200 x 10,000 pairs each, 10 closed-loop steps: 1739 us
+// with a CTA per 1024 B entries (2.1 an SM), six launches a step and a look-up
+// per 256 atoms; 1136 us now, 91 us of a step's 113 in the pair kernel.
 //
 // FP32_COMP grids only. The paper's bias routine is the serial counterpart
 // (one CPU rank), SI "Minimization of Interprocess Communications".
@@ -30,8 +39,10 @@ namespace abp {
 namespace {
 
 constexpr int kBigThreads = 256;
-constexpr int kBigJB = 4;
-constexpr int kBigChunk = kBigThreads * kBigJB;
+constexpr int kBigCnThreads = 64;  // k_big_cn: small CTAs, so that the last SM's share is small too
+constexpr int kBigJB = 6;  // B entries a thread (pair kernel, 32 x 200 x 10,000 pairs: 96.5 us with 4, 91 with 6)
+constexpr int kBigChunk = kBigCnThreads * kBigJB;
+constexpr int kBigForceThreads = 128;
 constexpr int kStencilPerBlock = 2048;
 
 __host__ __device__ constexpr int fixed_bytes_f() { return (int)((sizeof(GroupFixed<float>) + 31) & ~(size_t)31); }
@@ -41,8 +52,9 @@ __host__ __device__ inline size_t up256(size_t x) { return (x + 255) & ~(size_t)
 }  // namespace
 
 // Per-walker scratch of the phased form (in the walker's jscratch):
-//   BigHead | jA[na] | jB[nb] | part_s[nchunk][2] | part_g[nchunk][na][3]
-// for the walker's (single) COORD CV; jA/jB hold dCN/dx per list entry.
+//   BigHead | jA[na] | jB[nb] | a5 term tables
+// for the walker's (single) COORD CV; jA/jB hold dCN/dx per list entry. Its
+// CTAs' partial sums (in bpart): s[nchunk][2] | bad[nchunk] | g[nchunk][na][3].
 struct BigHead {
   float sh[kMaxCv], sl[kMaxCv];
   float com_u[kMaxCv][3];
@@ -51,6 +63,7 @@ struct BigHead {
   float df[kMaxCv];
   float hf;
   int dep, bad, flags;
+  float dv[kMaxCv];  // dV_b/ds after the step's deposits
   double h;
 };
 
@@ -66,21 +79,31 @@ __host__ __device__ inline int big_nchunks(const WalkerDev &wd) {
 }
 
 struct BigLayout {
-  size_t head, jA, jB, part_s, part_g, terms, nterm, total;
+  size_t head, jA, jB, terms, nterm, total;
 };
+
+struct BigParts {
+  float *s;   // [nchunk][2]
+  int *bad;   // [nchunk]
+  float *g;   // [nchunk][na][3]
+};
+__host__ __device__ inline BigParts big_parts(void *p, int nc) {
+  BigParts P;
+  P.s = static_cast<float *>(p);
+  P.bad = reinterpret_cast<int *>(P.s + 2 * nc);
+  P.g = reinterpret_cast<float *>(P.bad + nc);
+  return P;
+}
 
 __host__ __device__ inline BigLayout big_layout(const WalkerDev &wd) {
   BigLayout L;
   int k = big_cn_index(wd);
   int na = k < 0 ? 0 : wd.cv[k].na, nb = k < 0 ? 0 : wd.cv[k].nb;
-  int nc = big_nchunks(wd);
   L.head = 0;
   L.jA = up256(sizeof(BigHead));
   L.jB = L.jA + (size_t)na * 16;
-  L.part_s = up256(L.jB + (size_t)nb * 16);
-  L.part_g = up256(L.part_s + (size_t)nc * 8);
   // per atom, its a5 terms (big_atom_terms) and their count
-  L.terms = up256(L.part_g + (size_t)nc * na * 12);
+  L.terms = up256(L.jB + (size_t)nb * 16);
   L.nterm = up256(L.terms + (size_t)wd.natoms * kAtomTerms * 4);
   L.total = up256(L.nterm + (size_t)wd.natoms);
   return L;
@@ -116,6 +139,10 @@ int big_atom_terms(const WalkerDev &hd, const abp_walker_desc *d, std::vector<in
 }
 
 size_t big_scratch_bytes(const WalkerDev &hd) { return big_layout(hd).total; }
+size_t big_part_bytes(const WalkerDev &hd) {
+  const int k = big_cn_index(hd), nc = big_nchunks(hd);
+  return k < 0 ? 0 : (size_t)nc * (12 + (size_t)hd.cv[k].na * 12);
+}
 size_t big_terms_offset(const WalkerDev &hd) { return big_layout(hd).terms; }
 size_t big_nterm_offset(const WalkerDev &hd) { return big_layout(hd).nterm; }
 int big_cn_count(const WalkerDev &hd) {
@@ -136,180 +163,175 @@ __device__ __forceinline__ float min_image_rn(float d, float L, float invL) {
   return __fmaf_rn(-L, t, d);
 }
 
-// The A gradients of one block (4 A atoms x 3 components, this lane's part)
-// summed over the warp by a reduce-scatter: the half-warps exchange half of
-// the values (atoms 0, 1 | 2, 3), then the quarter-warps (one atom each),
-// then three butterfly levels over the remaining three; lane 8 q holds atom
-// q's sums, which it adds to the warp's accumulators.
-__device__ __forceinline__ void reduce_block_grads(const float (&gi)[4][3], int lane, int i0, int na, float *mylig) {
-  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
-  float w6[6];
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    const float lo = gi[j / 3][j % 3], hi = gi[2 + j / 3][j % 3];
-    const float send = h16 ? lo : hi;
-    w6[j] = (h16 ? hi : lo) + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-  float w3[3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    const float send = h8 ? w6[j] : w6[3 + j];
-    w3[j] = (h8 ? w6[3 + j] : w6[j]) + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) w3[j] += __shfl_xor_sync(0xffffffffu, w3[j], o);
-  const int ii = (h16 ? 2 : 0) + (h8 ? 1 : 0);
-  if ((lane & 7) == 0 && i0 + ii < na)
-#pragma unroll
-    for (int q = 0; q < 3; ++q) mylig[(i0 + ii) * 3 + q] += w3[q];
+// 1 / x for x >= 1 (infinity gives 0): one MUFU instruction.
+__device__ __forceinline__ float rcp_ge1(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
-// One CTA: the A x (one chunk of B) pairs of one walker's CN.
-__global__ void __launch_bounds__(kBigThreads) k_big_cn(const BigItem *items, const void *coords,
-                                                        const long long *coff, long long step_off) {
-  extern __shared__ __align__(32) unsigned char smem[];
-  const BigItem it = items[blockIdx.x];
+// The A gradients of a block of 8 A atoms (x 3 components, this lane's part)
+// summed over the warp by a reduce-scatter: three exchange levels halve the
+// atoms a lane keeps (8, 4, 2, 1), two more add the rest; lane 4 q holds atom
+// q's sums, which it stores.
+__device__ __forceinline__ void reduce_block_grads(float (&v)[24], int lane, int n, float *out) {
+#pragma unroll
+  for (int o = 16, m = 12; o >= 4; o >>= 1, m >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < 12; ++i)
+      if (i < m) {
+        const float keep = up ? v[m + i] : v[i], send = up ? v[i] : v[m + i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+  }
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+  const int q = lane >> 2;
+  if ((lane & 3) == 0 && q < n)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[3 * q + i] = v[i];
+}
+
+// A block of 8 A atoms (n of them valid) against the thread's kBigJB B
+// entries. MASK: pairs with an A or B atom past the end count nothing. The
+// switch values of an A atom, of at most kBigJB together, are added to a
+// compensated sum that starts at kBigJB (three additions give the exact error).
+template <bool PBC, bool MASK>
+__device__ __forceinline__ void big_block(const float4 *As, int n, const float (&xj)[kBigJB], const float (&yj)[kBigJB],
+                                          const float (&zj)[kBigJB], const float (&mj)[kBigJB], float (&gxj)[kBigJB],
+                                          float (&gyj)[kBigJB], float (&gzj)[kBigJB], float k2, const float *box,
+                                          const float *ibox, float &sacc, float &scomp, float (&gi)[24]) {
+#pragma unroll
+  for (int ii = 0; ii < 8; ++ii) {
+    const float4 a = As[MASK && ii >= n ? 0 : ii];
+    float g0 = 0.f, g1 = 0.f, g2 = 0.f, part = 0.f;
+#pragma unroll
+    for (int jj = 0; jj < kBigJB; ++jj) {
+      float dx = a.x - xj[jj], dy = a.y - yj[jj], dz = a.z - zj[jj];
+      if (PBC) {
+        dx = min_image_rn(dx, box[0], ibox[0]);
+        dy = min_image_rn(dy, box[1], ibox[1]);
+        dz = min_image_rn(dz, box[2], ibox[2]);
+      }
+      const float q = (dx * dx + dy * dy + dz * dz) * k2;
+      const float q2 = q * q;
+      float sw = rcp_ge1(__fmaf_rn(q2, q, 1.f));
+      if (MASK) sw *= ii < n ? mj[jj] : 0.f;
+      part += sw;
+      const float gf = q2 * (sw * sw);
+      g0 += gf * dx;
+      g1 += gf * dy;
+      g2 += gf * dz;
+      gxj[jj] += gf * dx;
+      gyj[jj] += gf * dy;
+      gzj[jj] += gf * dz;
+    }
+    const float t = __fadd_rn(sacc, part), z = __fsub_rn(t, sacc);
+    scomp = __fadd_rn(scomp, __fsub_rn(part, z));
+    sacc = t;
+    gi[3 * ii] = g0;
+    gi[3 * ii + 1] = g1;
+    gi[3 * ii + 2] = g2;
+  }
+}
+
+// One CTA: the A x (one chunk of B) pairs of one walker's CN. The A atoms are
+// read from shared memory, each thread holds kBigJB B entries and their
+// gradients. Bound by the FP32 issue: 18 operations a pair, 9 for a minimum
+// image, ~6 for the sums and exchanges.
+template <bool PBC>
+__device__ __forceinline__ void big_cn_body(const BigItem &it, const CvDev &c, const float4 *x, float4 *As, float *lig) {
   const WalkerDev *wd = it.wd;
-  const int k = big_cn_index(*wd);
-  const CvDev &c = wd->cv[k];
   const int na = c.na, nb = c.nb;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = kBigThreads / 32;
-  const float4 *x = reinterpret_cast<const float4 *>(coords) + coff[it.widx] + step_off;
-  float4 *As = reinterpret_cast<float4 *>(smem);
-  float *lig = reinterpret_cast<float *>(As + na);  // [nwarps][na][3]
-  for (int i = t; i < na; i += kBigThreads) As[i] = x[c.ia[i]];
-  for (int q = t; q < nwarps * na * 3; q += kBigThreads) lig[q] = 0.f;
-  __syncthreads();
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = kBigCnThreads / 32;
   const float k2 = (float)c.inv_r0sq, c6 = -6.f * k2;
-  const bool pbc = c.pbc != 0;
-  const float bx = (float)c.box[0], by = (float)c.box[1], bz = (float)c.box[2];
-  const float ibx = (float)c.inv_box[0], iby = (float)c.inv_box[1], ibz = (float)c.inv_box[2];
+  const float box[3] = {(float)c.box[0], (float)c.box[1], (float)c.box[2]};
+  const float ibox[3] = {(float)c.inv_box[0], (float)c.inv_box[1], (float)c.inv_box[2]};
   const int j0 = it.chunk * kBigChunk;
   float xj[kBigJB], yj[kBigJB], zj[kBigJB], gxj[kBigJB], gyj[kBigJB], gzj[kBigJB], mj[kBigJB];
 #pragma unroll
   for (int jj = 0; jj < kBigJB; ++jj) {
-    int j = j0 + jj * kBigThreads + t;
-    bool ok = j < nb;
-    float4 p = x[c.ib[ok ? j : 0]];
+    const int j = j0 + jj * kBigCnThreads + t;
+    const bool ok = j < nb;
+    const float4 p = x[c.ib[ok ? j : 0]];
     xj[jj] = p.x;
     yj[jj] = p.y;
     zj[jj] = p.z;
     mj[jj] = ok ? 1.f : 0.f;
     gxj[jj] = gyj[jj] = gzj[jj] = 0.f;
   }
-  // the thread's CN terms: each block of 4 A atoms x kBigJB B entries summed
-  // in (A, B) order, the block's sum added to a compensated (two-sum)
-  // accumulator
-  float sacc = 0.f, scomp = 0.f;
+  float sacc = (float)kBigJB, scomp = 0.f;
   float *mylig = lig + warp * na * 3;
-  // every B entry of this CTA in range: blocks of 4 A atoms need no mask
-  // (a mask of 1 would change no bit)
-  const bool fullj = j0 + kBigJB * kBigThreads <= nb;
-  for (int i0 = 0; i0 < na; i0 += 4) {
-    float gi[4][3];
-    float part = 0.f;
-    if (fullj && i0 + 4 <= na) {
-#pragma unroll
-      for (int ii = 0; ii < 4; ++ii) {
-        gi[ii][0] = gi[ii][1] = gi[ii][2] = 0.f;
-        float4 a = As[i0 + ii];
-#pragma unroll
-        for (int jj = 0; jj < kBigJB; ++jj) {
-          float dx = a.x - xj[jj], dy = a.y - yj[jj], dz = a.z - zj[jj];
-          if (pbc) {
-            dx = min_image_rn(dx, bx, ibx);
-            dy = min_image_rn(dy, by, iby);
-            dz = min_image_rn(dz, bz, ibz);
-          }
-          float q = (dx * dx + dy * dy + dz * dz) * k2;
-          float q2 = q * q;
-          float sw = __fdividef(1.f, 1.f + q2 * q);
-          part += sw;
-          float gf = c6 * q2 * sw * sw;
-          gi[ii][0] += gf * dx;
-          gi[ii][1] += gf * dy;
-          gi[ii][2] += gf * dz;
-          gxj[jj] -= gf * dx;
-          gyj[jj] -= gf * dy;
-          gzj[jj] -= gf * dz;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int ii = 0; ii < 4; ++ii) {
-        gi[ii][0] = gi[ii][1] = gi[ii][2] = 0.f;
-        int i = i0 + ii;
-        bool oki = i < na;
-        float4 a = As[oki ? i : 0];
-#pragma unroll
-        for (int jj = 0; jj < kBigJB; ++jj) {
-          float dx = a.x - xj[jj], dy = a.y - yj[jj], dz = a.z - zj[jj];
-          if (pbc) {
-            dx = min_image_rn(dx, bx, ibx);
-            dy = min_image_rn(dy, by, iby);
-            dz = min_image_rn(dz, bz, ibz);
-          }
-          float q = (dx * dx + dy * dy + dz * dz) * k2;
-          float q2 = q * q;
-          float sw = __fdividef(1.f, 1.f + q2 * q);
-          float m = oki ? mj[jj] : 0.f;
-          part += m * sw;
-          float gf = c6 * m * q2 * sw * sw;
-          gi[ii][0] += gf * dx;
-          gi[ii][1] += gf * dy;
-          gi[ii][2] += gf * dz;
-          gxj[jj] -= gf * dx;
-          gyj[jj] -= gf * dy;
-          gzj[jj] -= gf * dz;
-        }
-      }
-    }
-    {
-      float tsum, terr;
-      two_sum<float>(sacc, part, tsum, terr);
-      sacc = tsum;
-      scomp += terr;
-    }
-    reduce_block_grads(gi, lane, i0, na, mylig);
+  const bool fullj = j0 + kBigChunk <= nb;
+  for (int i0 = 0; i0 < na; i0 += 8) {
+    const int n = min(8, na - i0);
+    float gi[24];
+    if (fullj && n == 8)
+      big_block<PBC, false>(As + i0, n, xj, yj, zj, mj, gxj, gyj, gzj, k2, box, ibox, sacc, scomp, gi);
+    else
+      big_block<PBC, true>(As + i0, n, xj, yj, zj, mj, gxj, gyj, gzj, k2, box, ibox, sacc, scomp, gi);
+    reduce_block_grads(gi, lane, n, mylig + 3 * i0);
   }
-  unsigned char *js = reinterpret_cast<unsigned char *>(wd->jscratch);
   const BigLayout L = big_layout(*wd);
-  float4 *jB = reinterpret_cast<float4 *>(js + L.jB);
+  const BigParts P = big_parts(wd->bpart, big_nchunks(*wd));
+  float4 *jB = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(wd->jscratch) + L.jB);
 #pragma unroll
   for (int jj = 0; jj < kBigJB; ++jj) {
-    int j = j0 + jj * kBigThreads + t;
-    if (j < nb) jB[j] = make_float4(gxj[jj], gyj[jj], gzj[jj], 0.f);
+    const int j = j0 + jj * kBigCnThreads + t;
+    if (j < nb) jB[j] = make_float4(-c6 * gxj[jj], -c6 * gyj[jj], -c6 * gzj[jj], 0.f);
   }
-  // this chunk's CN as hi + lo: warps in order, lanes by butterfly
-  float sh, sl;
-  two_sum<float>(sacc, scomp, sh, sl);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
-    ff_add<float>(sh, sl, oh, ol);
-  }
-  // (every lane now holds the same pair: the pairwise add is commutative)
-  __shared__ float wsum[kBigThreads / 32][2];
+  // this chunk's CN as hi + lo: lanes by butterfly, warps in order
+  float h[1], l[1];
+  two_sum<float>(__fsub_rn(sacc, (float)kBigJB), scomp, h[0], l[0]);
+  warp_sum_ff<1>(h, l);
+  __shared__ float wsum[kBigCnThreads / 32][2];
   if (lane == 0) {
-    wsum[warp][0] = sh;
-    wsum[warp][1] = sl;
+    wsum[warp][0] = h[0];
+    wsum[warp][1] = l[0];
   }
   __syncthreads();
-  float *part_s = reinterpret_cast<float *>(js + L.part_s) + 2 * it.chunk;
   if (t == 0) {
-    float h = wsum[0][0], l = wsum[0][1];
-    for (int w = 1; w < nwarps; ++w) ff_add<float>(h, l, wsum[w][0], wsum[w][1]);
-    part_s[0] = h;
-    part_s[1] = l;
+    float sh = wsum[0][0], sl = wsum[0][1];
+    for (int w = 1; w < nwarps; ++w) ff_add<float>(sh, sl, wsum[w][0], wsum[w][1]);
+    P.s[2 * it.chunk] = sh;
+    P.s[2 * it.chunk + 1] = sl;
   }
-  float *part_g = reinterpret_cast<float *>(js + L.part_g) + (size_t)it.chunk * na * 3;
-  for (int q = t; q < na * 3; q += kBigThreads) {
-    float acc = 0.f;
-    for (int w = 0; w < nwarps; ++w) acc += lig[w * na * 3 + q];
-    part_g[q] = acc;
+  float *part_g = P.g + (size_t)it.chunk * na * 3;
+  for (int q = t; q < na * 3; q += kBigCnThreads) {
+    float acc = lig[q];
+    for (int w = 1; w < nwarps; ++w) acc += lig[w * na * 3 + q];
+    part_g[q] = c6 * acc;
   }
+}
+
+__global__ void __launch_bounds__(kBigCnThreads, 6) k_big_cn(const BigItem *items, const void *coords,
+                                                          const long long *coff, long long step_off) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  const BigItem it = items[blockIdx.x];
+  const WalkerDev *wd = it.wd;
+  const CvDev &c = wd->cv[big_cn_index(*wd)];
+  chain_wait();
+  const float4 *x = reinterpret_cast<const float4 *>(coords) + coff[it.widx] + step_off;
+  float4 *As = reinterpret_cast<float4 *>(smem);
+  float *lig = reinterpret_cast<float *>(As + c.na);  // [warps][na][3]
+  for (int i = threadIdx.x; i < c.na; i += kBigCnThreads) As[i] = x[c.ia[i]];
+  // this CTA's share of the walker's atoms: all finite?
+  const int nc = big_nchunks(*wd);
+  const int lo = (int)((long long)wd->natoms * it.chunk / nc), hi = (int)((long long)wd->natoms * (it.chunk + 1) / nc);
+  int bad = 0;
+  for (int i = lo + (int)threadIdx.x; i < hi; i += kBigCnThreads) {
+    const float4 p = x[i];
+    bad |= (isfinite(p.x) && isfinite(p.y) && isfinite(p.z)) ? 0 : 1;
+  }
+  bad = __syncthreads_or(bad);  // (and the A atoms are in place)
+  if (threadIdx.x == 0) big_parts(wd->bpart, nc).bad[it.chunk] = bad;
+  if (c.pbc)
+    big_cn_body<true>(it, c, x, As, lig);
+  else
+    big_cn_body<false>(it, c, x, As, lig);
 }
 
 // ---------------------------------------------------------------- k_big_cvs
@@ -344,14 +366,14 @@ __device__ void big_load_desc(const Grp &g, GroupFixed<float> *fx, const WalkerD
   g.sync();
 }
 
-// Centre-of-mass distance with compensated arithmetic: each weighted offset
-// w (x - r_G) is split exactly into hi + lo (the difference by two_sum, the
-// product's error by fma; w times the difference's low part, tiny, rounded
-// once), summed as hi + lo pairs, and |d| is taken in hi + lo. Groups spread
-// over a large box (as a group of environment atoms is) otherwise lose the
-// ~1e-8 relative accuracy a hill a few grid spacings wide needs.
-__device__ void cv_com_ff(const Grp &g, GroupFixed<float> *fx, int k, const float4 *xs) {
-  const CvDev &c = fx->wd.cv[k];
+// Centre-of-mass distance with compensated arithmetic, by the whole CTA: each
+// weighted offset w (x - r_G) is split exactly into hi + lo (the difference by
+// two_sum, the product's error by fma; w times the difference's low part,
+// tiny, rounded once), summed as hi + lo pairs, and |d| is taken in hi + lo
+// (com_finish_ff). Groups spread over a large box (as a group of environment
+// atoms is) otherwise lose the ~1e-8 relative accuracy a hill a few grid
+// spacings wide needs. Part 1: every warp's sums to part[warp][6][2].
+__device__ __forceinline__ void big_com_part(const Grp &g, const CvDev &c, const float4 *xs, float (*part)[6][2]) {
   const float4 ra = xs[c.ia[0]], rb = xs[c.ib[0]];
   float h[6] = {0, 0, 0, 0, 0, 0}, l[6] = {0, 0, 0, 0, 0, 0};
   auto acc = [&](int q, float w, float x, float r) {
@@ -375,71 +397,83 @@ __device__ void cv_com_ff(const Grp &g, GroupFixed<float> *fx, int k, const floa
     acc(4, w, p.y, rb.y);
     acc(5, w, p.z, rb.z);
   }
-  for (int q = 0; q < 6; ++q) grp_sum_ff<float>(g, h[q], l[q], fx->red);
-  if (g.t != 0) return;
-  // equal masses: the weights' FP32 rounding, one factor per group
-  for (int q = 0; q < 3; ++q) {
-    if (c.wc_a != 0.f) ff_add<float>(h[q], l[q], __fmul_rn(h[q], c.wc_a), 0.f);
-    if (c.wc_b != 0.f) ff_add<float>(h[3 + q], l[3 + q], __fmul_rn(h[3 + q], c.wc_b), 0.f);
-  }
-  float dh[3], dl[3];
-  const float ra3[3] = {ra.x, ra.y, ra.z}, rb3[3] = {rb.x, rb.y, rb.z};
-  for (int q = 0; q < 3; ++q) {
-    float rdh, rdl;  // r_B - r_A exactly, as hi + lo
-    two_sum<float>(rb3[q], -ra3[q], rdh, rdl);
-    float s, e;
-    two_sum<float>(rdh, h[3 + q], s, e);
-    e += l[3 + q] + rdl;
-    float s2, e2;
-    two_sum<float>(s, -h[q], s2, e2);
-    e2 += e - l[q];
-    dh[q] = s2 + e2;
-    dl[q] = e2 - (dh[q] - s2);
-    if (c.pbc) {
-      float shift = (float)c.box[q] * floor(dh[q] * (float)c.inv_box[q] + 0.5f);
-      float t, te;
-      two_sum<float>(dh[q], -shift, t, te);
-      dh[q] = t;
-      dl[q] += te;
+  warp_sum_ff<6>(h, l);
+  if (g.lane == 0)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      part[g.warp][q][0] = h[q];
+      part[g.warp][q][1] = l[q];
     }
+}
+// Part 2, by one warp: lane q < 6 adds the warps' sums of component q in warp
+// order, lane 0 finishes.
+__device__ __forceinline__ void big_com_end(const Grp &g, GroupFixed<float> *fx, int k, const float4 *xs,
+                                            const float (*part)[6][2]) {
+  const CvDev &c = fx->wd.cv[k];
+  float h = 0.f, l = 0.f;
+  if (g.lane < 6)
+    for (int w = 0; w < g.nwarps; ++w) ff_add<float>(h, l, part[w][g.lane][0], part[w][g.lane][1]);
+  float hh[6], ll[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    hh[q] = __shfl_sync(0xffffffffu, h, q);
+    ll[q] = __shfl_sync(0xffffffffu, l, q);
   }
-  // r^2 = sum (dh + dl)^2 in hi + lo, then r = sqrt with one Newton correction
-  float r2h = 0, r2l = 0;
-  for (int q = 0; q < 3; ++q) {
-    float p = dh[q] * dh[q];
-    float e = fmaf(dh[q], dh[q], -p) + 2.f * dh[q] * dl[q];
-    ff_add<float>(r2h, r2l, p, e);
-  }
-  float rh = sqrtf(r2h);
-  float rl = rh > 0 ? (fmaf(-rh, rh, r2h) + r2l) / (2.f * rh) : 0.f;
-  fx->sh[k] = rh;
-  fx->sl[k] = rl;
-  if (rh > 0) {
-    float ir = 1.f / rh;
-    for (int q = 0; q < 3; ++q) fx->com_u[k][q] = dh[q] * ir;
-  } else {
-    for (int q = 0; q < 3; ++q) fx->com_u[k][q] = 0;
-    fx->flags |= ABP_WFLAG_SINGULAR;
+  if (g.lane != 0) return;
+  const float4 ra = xs[c.ia[0]], rb = xs[c.ib[0]];
+  const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
+  float s, sl;
+  const int fl = com_finish_ff(c, a0, hh, ll, b0, hh + 3, ll + 3, s, sl, fx->com_u[k]);
+  fx->sh[k] = s;
+  fx->sl[k] = sl;
+  if (fl) atomicOr(&fx->flags, fl);
+}
+
+// a4 of a walker whose CVs are in fx: V and dV/ds to its head and state.
+__device__ __forceinline__ void big_lookup(const Grp &g, GroupFixed<float> *fx, BigHead *head, long long step) {
+  const GroupLayout none{};
+  interp_step<float, false>(g, fx, none, nullptr);
+  const WalkerDev &wd = fx->wd;
+  if (g.t == 0) {
+    for (int k = 0; k < kMaxCv; ++k) head->dv[k] = k < wd.g.d ? fx->dvds[k] : 0.f;
+    WalkerState st;
+    for (int k = 0; k < 3; ++k) {
+      st.s[k] = k < wd.g.d ? (double)fx->sh[k] + (double)fx->sl[k] : 0.0;
+      st.dV[k] = k < wd.g.d ? (double)fx->dV[k] : 0.0;
+    }
+    st.V = (double)fx->V;
+    st.flags = fx->flags;
+    st.pad = 0;
+    st.step = step;
+    *wd.state = st;
   }
 }
 
-// One CTA per walker: CVs, axis state, height; hill record to the head.
+// One CTA per walker: CVs, axis state, height; hill record to the head; with
+// `look` (no walker deposits this step) the look-up too.
 __global__ void __launch_bounds__(kBigThreads) k_big_cvs(const BigItem *walkers, const void *coords,
                                                          const long long *coff, long long step_off, long long step,
-                                                         DepositLog log, DevCounters *ctr) {
+                                                         DepositLog log, DevCounters *ctr, int look) {
   extern __shared__ __align__(32) unsigned char smem[];
   Grp g = big_group();
   GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
   const BigItem it = walkers[blockIdx.x];
   big_load_desc(g, fx, it.wd);
+  chain_wait();
   const WalkerDev &wd = fx->wd;
   const float4 *x = reinterpret_cast<const float4 *>(coords) + coff[it.widx] + step_off;
   unsigned char *js = reinterpret_cast<unsigned char *>(wd.jscratch);
   BigHead *head = reinterpret_cast<BigHead *>(js);
+  const int kc = big_cn_index(wd), nc = big_nchunks(wd);
+  const BigParts P = big_parts(wd.bpart, nc);
   int bad = 0;
-  for (int i = g.t; i < wd.natoms; i += g.G) {
-    float4 p = x[i];
-    bad |= (isfinite(p.x) && isfinite(p.y) && isfinite(p.z)) ? 0 : 1;
+  if (nc > 0) {  // the pair kernel's CTAs looked at every atom
+    for (int q = g.t; q < nc; q += g.G) bad |= P.bad[q];
+  } else {
+    for (int i = g.t; i < wd.natoms; i += g.G) {
+      float4 p = x[i];
+      bad |= (isfinite(p.x) && isfinite(p.y) && isfinite(p.z)) ? 0 : 1;
+    }
   }
   if (grp_any<float>(g, fx, bad)) {
     if (g.t == 0) {
@@ -450,39 +484,49 @@ __global__ void __launch_bounds__(kBigThreads) k_big_cvs(const BigItem *walkers,
     }
     return;
   }
-  const BigLayout L = big_layout(wd);
-  const int kc = big_cn_index(wd);
-  for (int k = 0; k < wd.g.d; ++k) {
-    const CvDev &c = wd.cv[k];
-    if (c.type == ABP_CV_COM_DIST) {
-      cv_com_ff(g, fx, k, x);
-    } else if (c.type == ABP_CV_DIHEDRAL) {
-      cv_dihedral<float>(g, fx, k, x);
+  // COM distances on every warp, a dihedral on the last warp's last lane, the
+  // CN's partial sums on the second warp
+  __shared__ float part[kMaxCv][kBigThreads / 32][6][2];
+  for (int k = 0; k < wd.g.d; ++k)
+    if (wd.cv[k].type == ABP_CV_COM_DIST) big_com_part(g, wd.cv[k], x, part[k]);
+  for (int k = 0; k < wd.g.d; ++k)
+    if (wd.cv[k].type == ABP_CV_DIHEDRAL) cv_dihedral<float>(g, fx, k, x);
+  if (kc >= 0 && g.warp == 1) {
+    float h[1] = {0.f}, l[1] = {0.f};
+    for (int q = g.lane; q < nc; q += 32) ff_add<float>(h[0], l[0], P.s[2 * q], P.s[2 * q + 1]);
+    warp_sum_ff<1>(h, l);
+    if (g.lane == 0) {
+      fx->sh[kc] = h[0];
+      fx->sl[kc] = l[0];
     }
   }
-  if (kc >= 0) {
-    const CvDev &c = wd.cv[kc];
-    const int nc = big_nchunks(wd);
-    const float *part_s = reinterpret_cast<const float *>(js + L.part_s);
-    const float *part_g = reinterpret_cast<const float *>(js + L.part_g);
-    if (g.t == 0) {
-      float h = part_s[0], l = part_s[1];
-      for (int q = 1; q < nc; ++q) ff_add<float>(h, l, part_s[2 * q], part_s[2 * q + 1]);
-      fx->sh[kc] = h;
-      fx->sl[kc] = l;
-    }
-    float4 *jA = reinterpret_cast<float4 *>(js + L.jA);
-    for (int i = g.t; i < c.na; i += g.G) {
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-      for (int q = 0; q < nc; ++q) {
-        const float *p = part_g + ((size_t)q * c.na + i) * 3;
-        a0 += p[0];
-        a1 += p[1];
-        a2 += p[2];
+  g.sync();
+  if (kc >= 0 && g.warp >= 2) {
+    // A gradients: the CTAs' sums in chunk order, NQ components a thread (not needed before a5)
+    float *jA = reinterpret_cast<float *>(js + big_layout(wd).jA);
+    constexpr int NQ = 4;
+    const int n3 = wd.cv[kc].na * 3, T = g.G - 64;
+    for (int q0 = g.t - 64; q0 < n3; q0 += NQ * T) {
+      float acc[NQ];
+#pragma unroll
+      for (int u = 0; u < NQ; ++u) acc[u] = 0.f;
+#pragma unroll 9
+      for (int w = 0; w < nc; ++w)
+#pragma unroll
+        for (int u = 0; u < NQ; ++u) {
+          const int q = q0 + u * T;
+          if (q < n3) acc[u] += P.g[(size_t)w * n3 + q];
+        }
+#pragma unroll
+      for (int u = 0; u < NQ; ++u) {
+        const int q = q0 + u * T;
+        if (q < n3) jA[(q / 3) * 4 + q % 3] = acc[u];
       }
-      jA[i] = make_float4(a0, a1, a2, 0.f);
     }
   }
+  if (g.warp == 0)
+    for (int k = 0; k < wd.g.d; ++k)
+      if (wd.cv[k].type == ABP_CV_COM_DIST) big_com_end(g, fx, k, x, part[k]);
   g.sync();
   const bool dep = (step % wd.stride) == 0;
   if (g.t < wd.g.d) axis_setup<float>(fx, g.t, dep);
@@ -537,7 +581,8 @@ __global__ void __launch_bounds__(kBigThreads) k_big_cvs(const BigItem *walkers,
   if (g.t == 0) {
     head->bad = 0;
     head->dep = dep ? 1 : 0;
-    head->flags = fx->flags | (dep ? ABP_WFLAG_DEPOSIT : 0);
+    if (dep) fx->flags |= ABP_WFLAG_DEPOSIT;
+    head->flags = fx->flags;
     for (int k = 0; k < kMaxCv; ++k) {
       head->sh[k] = fx->sh[k];
       head->sl[k] = fx->sl[k];
@@ -550,6 +595,8 @@ __global__ void __launch_bounds__(kBigThreads) k_big_cvs(const BigItem *walkers,
         for (int q = 0; q < 3; ++q) head->dih_g[k][a][q] = fx->dih_g[k][a][q];
     }
   }
+  g.sync();
+  if (look) big_lookup(g, fx, head, step);
 }
 
 // ---------------------------------------------------------------- deposit + refresh
@@ -575,6 +622,7 @@ __global__ void __launch_bounds__(kBigThreads) k_big_deposit(const BigItem *walk
   extern __shared__ __align__(32) unsigned char smem[];
   Grp g = big_group();
   GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
+  chain_wait();
   if (!big_tables(g, fx, walkers[blockIdx.x])) return;
   const WalkerDev &wd = fx->wd;
   const GridDev &gd = wd.g;
@@ -611,6 +659,7 @@ __global__ void __launch_bounds__(kBigThreads) k_big_refresh(const BigItem *walk
   extern __shared__ __align__(32) unsigned char smem[];
   Grp g = big_group();
   GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
+  chain_wait();
   if (!big_tables(g, fx, walkers[blockIdx.x])) return;
   const WalkerDev &wd = fx->wd;
   const GridDev &gd = wd.g;
@@ -645,143 +694,124 @@ __global__ void __launch_bounds__(kBigThreads) k_big_refresh(const BigItem *walk
   }
 }
 
+// ---------------------------------------------------------------- a4 after deposits
+
+// One warp per walker: the look-up after the step's deposits.
+__global__ void __launch_bounds__(32) k_big_lookup(const BigItem *walkers, long long step) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  const Grp g = big_group();
+  GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
+  big_load_desc(g, fx, walkers[blockIdx.x].wd);
+  chain_wait();
+  BigHead *head = reinterpret_cast<BigHead *>(fx->wd.jscratch);
+  if (head->bad) return;
+  if (g.t < kMaxCv) {
+    fx->sh[g.t] = head->sh[g.t];
+    fx->sl[g.t] = head->sl[g.t];
+  }
+  if (g.t == 0) fx->flags = head->flags;
+  g.sync();
+  if (g.t < fx->wd.g.d) axis_setup<float>(fx, g.t, false);
+  g.sync();
+  big_lookup(g, fx, head, step);
+}
+
 // ---------------------------------------------------------------- k_big_force
 
-// a4 + a5 of one walker's atoms [blockIdx.x * kBigThreads, + kBigThreads):
-// each CTA forms the walker's dV/ds (a few corner reads), then each thread
-// sums its atom's terms in the walker's fixed order (CV by CV, list A before
-// list B) and writes the walker's force buffer and, when given, the
-// caller's.
-__global__ void __launch_bounds__(kBigThreads) k_big_force(const BigItem *walkers, void *forces,
-                                                           const long long *foff, long long force_step_off, int mode,
-                                                           long long step) {
-  extern __shared__ __align__(32) unsigned char smem[];
-  Grp g = big_group();
-  GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
+// a5 of one walker's atoms [blockIdx.x * kBigForceThreads, + kBigForceThreads):
+// each thread sums its atom's terms in the walker's fixed order (CV by CV,
+// list A before list B) and writes the walker's force buffer and, when given,
+// the caller's. Closed loop (move): it then moves the atom, x += c1
+// F_bias + c2 xi (this form takes no CV potential), the coordinates before
+// the move to the trajectory records when given. A walker whose step saw
+// non-finite coordinates gets no force and does not move.
+__global__ void __launch_bounds__(kBigForceThreads) k_big_force(const BigItem *walkers, void *forces,
+                                                                const long long *foff, long long force_step_off,
+                                                                int mode, long long step, MdParams md, int move,
+                                                                void *xio, const long long *coff, void *traj,
+                                                                const long long *toff, long long traj_step_off) {
   const BigItem it = walkers[blockIdx.y];
-  const int i0 = blockIdx.x * kBigThreads;
-  if (i0 >= it.wd->natoms) return;  // the whole CTA: past this walker's atoms
-  big_load_desc(g, fx, it.wd);
-  const WalkerDev &wd = fx->wd;
+  const WalkerDev &wd = *it.wd;
+  const int i = blockIdx.x * kBigForceThreads + threadIdx.x;
+  float n[3] = {0.f, 0.f, 0.f};
+  if (move && i < wd.natoms) md_normals(md.seed, it.stream, step, i, n);  // needs no earlier result
+  chain_wait();
+  if (i >= wd.natoms) return;
   unsigned char *js = reinterpret_cast<unsigned char *>(wd.jscratch);
   const BigHead *head = reinterpret_cast<const BigHead *>(js);
   float4 *fb = reinterpret_cast<float4 *>(wd.fbuf);
   float4 *fo = forces ? reinterpret_cast<float4 *>(forces) + foff[it.widx] + force_step_off : fb;
   const int fmode = forces ? mode : ABP_FORCES_OVERWRITE;
-  const int i = i0 + g.t;
   if (head->bad) {
-    if (fmode == ABP_FORCES_OVERWRITE && i < wd.natoms) fo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (blockIdx.x == 0 && g.t == 0) wd.state->flags = ABP_WFLAG_NONFINITE;
+    if (fmode == ABP_FORCES_OVERWRITE) fo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i == 0) wd.state->flags = ABP_WFLAG_NONFINITE;
     return;
   }
-  if (g.t < kMaxCv) {
-    fx->sh[g.t] = head->sh[g.t];
-    fx->sl[g.t] = head->sl[g.t];
-    for (int q = 0; q < 3; ++q) fx->com_u[g.t][q] = head->com_u[g.t][q];
-    for (int a = 0; a < 4; ++a)
-      for (int q = 0; q < 3; ++q) fx->dih_g[g.t][a][q] = head->dih_g[g.t][a][q];
-  }
-  if (g.t == 0) fx->flags = head->flags;
-  g.sync();
-  if (g.t < wd.g.d) axis_setup<float>(fx, g.t, false);
-  g.sync();
-  GroupLayout Ldummy{};
-  interp_step<float, false>(g, fx, Ldummy, nullptr);
-  if (i < wd.natoms) {
-    const BigLayout L = big_layout(wd);
-    const int32_t *tt = reinterpret_cast<const int32_t *>(js + L.terms) + (size_t)i * kAtomTerms;
-    const int ne = js[L.nterm + i];
-    const float4 *jA = reinterpret_cast<const float4 *>(js + L.jA);
-    const float4 *jB = reinterpret_cast<const float4 *>(js + L.jB);
-    float f0 = 0.f, f1 = 0.f, f2 = 0.f;
-    for (int q = 0; q < ne; ++q) {
-      const int code = tt[q], kind = code & 7, k = (code >> 3) & 3, pos = code >> 5;
-      const float dv = fx->dvds[k];
-      if (kind == kTermComA || kind == kTermComB) {
-        const float ux = fx->com_u[k][0] * dv, uy = fx->com_u[k][1] * dv, uz = fx->com_u[k][2] * dv;
-        if (kind == kTermComA) {
-          const float w = wd.cv[k].wa[pos];
-          f0 += w * ux;
-          f1 += w * uy;
-          f2 += w * uz;
-        } else {
-          const float w = wd.cv[k].wb[pos];
-          f0 -= w * ux;
-          f1 -= w * uy;
-          f2 -= w * uz;
-        }
-      } else if (kind == kTermDih) {
-        f0 -= dv * fx->dih_g[k][pos][0];
-        f1 -= dv * fx->dih_g[k][pos][1];
-        f2 -= dv * fx->dih_g[k][pos][2];
+  const BigLayout L = big_layout(wd);
+  const int32_t *tt = reinterpret_cast<const int32_t *>(js + L.terms) + (size_t)i * kAtomTerms;
+  const int ne = js[L.nterm + i];
+  const float4 *jA = reinterpret_cast<const float4 *>(js + L.jA);
+  const float4 *jB = reinterpret_cast<const float4 *>(js + L.jB);
+  float f0 = 0.f, f1 = 0.f, f2 = 0.f;
+  for (int q = 0; q < ne; ++q) {
+    const int code = tt[q], kind = code & 7, k = (code >> 3) & 3, pos = code >> 5;
+    const float dv = head->dv[k];
+    if (kind == kTermComA || kind == kTermComB) {
+      const float ux = head->com_u[k][0] * dv, uy = head->com_u[k][1] * dv, uz = head->com_u[k][2] * dv;
+      if (kind == kTermComA) {
+        const float w = wd.cv[k].wa[pos];
+        f0 += w * ux;
+        f1 += w * uy;
+        f2 += w * uz;
       } else {
-        const float4 j = kind == kTermCnA ? jA[pos] : jB[pos];
-        f0 -= dv * j.x;
-        f1 -= dv * j.y;
-        f2 -= dv * j.z;
+        const float w = wd.cv[k].wb[pos];
+        f0 -= w * ux;
+        f1 -= w * uy;
+        f2 -= w * uz;
       }
-    }
-    fb[i] = make_float4(f0, f1, f2, 0.f);
-    if (fo != fb) {
-      if (fmode == ABP_FORCES_ACCUMULATE) {
-        float4 o = fo[i];
-        o.x += f0;
-        o.y += f1;
-        o.z += f2;
-        fo[i] = o;
-      } else {
-        fo[i] = make_float4(f0, f1, f2, 0.f);
-      }
+    } else if (kind == kTermDih) {
+      f0 -= dv * head->dih_g[k][pos][0];
+      f1 -= dv * head->dih_g[k][pos][1];
+      f2 -= dv * head->dih_g[k][pos][2];
+    } else {
+      const float4 j = kind == kTermCnA ? jA[pos] : jB[pos];
+      f0 -= dv * j.x;
+      f1 -= dv * j.y;
+      f2 -= dv * j.z;
     }
   }
-  if (blockIdx.x == 0 && g.t == 0) {
-    WalkerState st;
-    for (int k = 0; k < 3; ++k) {
-      st.s[k] = k < wd.g.d ? (double)fx->sh[k] + (double)fx->sl[k] : 0.0;
-      st.dV[k] = k < wd.g.d ? (double)fx->dV[k] : 0.0;
+  fb[i] = make_float4(f0, f1, f2, 0.f);
+  if (fo != fb) {
+    if (fmode == ABP_FORCES_ACCUMULATE) {
+      float4 o = fo[i];
+      o.x += f0;
+      o.y += f1;
+      o.z += f2;
+      fo[i] = o;
+    } else {
+      fo[i] = make_float4(f0, f1, f2, 0.f);
     }
-    st.V = (double)fx->V;
-    st.flags = fx->flags;
-    st.pad = 0;
-    st.step = step;
-    *wd.state = st;
   }
-}
-
-// ---------------------------------------------------------------- k_big_move
-
-// Closed loop (abp_md_run): after the force phase, the move of one walker's
-// atoms [blockIdx.x * kBigThreads, + kBigThreads): x += c1 F_bias + c2 xi
-// (this form takes no CV potential), the coordinates before the move to the
-// trajectory records when given. A walker whose step saw non-finite
-// coordinates does not move.
-__global__ void __launch_bounds__(kBigThreads) k_big_move(const BigItem *walkers, MdParams md, void *xio,
-                                                          const long long *coff, void *traj, const long long *toff,
-                                                          long long traj_step_off, long long step) {
-  const BigItem it = walkers[blockIdx.y];
-  const WalkerDev *wd = it.wd;
-  const int i = blockIdx.x * kBigThreads + threadIdx.x;
-  if (i >= wd->natoms) return;
-  const BigHead *head = reinterpret_cast<const BigHead *>(wd->jscratch);
-  if (head->bad) return;
-  float4 *x = reinterpret_cast<float4 *>(xio) + coff[it.widx] + i;
-  const float4 f = reinterpret_cast<const float4 *>(wd->fbuf)[i];
-  float4 p = *x;
-  if (traj) reinterpret_cast<float4 *>(traj)[toff[it.widx] + traj_step_off + i] = p;
-  float n[3];
-  md_normals(md.seed, it.stream, step, i, n);
-  const float c1 = (float)md.c1, c2 = (float)md.c2;
-  p.x += c1 * f.x + c2 * n[0];
-  p.y += c1 * f.y + c2 * n[1];
-  p.z += c1 * f.z + c2 * n[2];
-  *x = p;
+  if (move) {
+    float4 *x = reinterpret_cast<float4 *>(xio) + coff[it.widx] + i;
+    float4 p = *x;
+    if (traj) reinterpret_cast<float4 *>(traj)[toff[it.widx] + traj_step_off + i] = p;
+    const float c1 = (float)md.c1, c2 = (float)md.c2;
+    p.x += c1 * f0 + c2 * n[0];
+    p.y += c1 * f1 + c2 * n[1];
+    p.z += c1 * f2 + c2 * n[2];
+    *x = p;
+  }
 }
 
 // ---------------------------------------------------------------- launcher
 
 cudaError_t launch_big_step(const BigArgs &a, cudaStream_t st) {
   const size_t fixed = (size_t)fixed_bytes_f();
-  const int ph = a.phases ? a.phases : 31;
+  // all phases: without a deposit this step the grid does not change, and the
+  // look-up goes with the CVs
+  const bool look = !a.phases && !a.any_deposit;
+  const int ph = a.phases ? a.phases : a.any_deposit ? 31 : 19;
   LaunchTimer *tm = a.timer;
   auto t0 = [&](const char *k) {
     nvtxRangePushA(k);
@@ -791,41 +821,49 @@ cudaError_t launch_big_step(const BigArgs &a, cudaStream_t st) {
     if (tm) tm->end(k, st);
     nvtxRangePop();
   };
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   if ((ph & 1) && a.ncn_items > 0) {
     e = smem_attr(reinterpret_cast<const void *>(k_big_cn), a.cn_smem);
     if (e != cudaSuccess) return e;
     t0("k_big_cn");
-    k_big_cn<<<a.ncn_items, kBigThreads, a.cn_smem, st>>>(a.cn_items, a.coords, a.coff, a.step_off);
+    e = launch_chained(k_big_cn, a.ncn_items, kBigCnThreads, a.cn_smem, st, a.cn_items, a.coords, a.coff, a.step_off);
+    if (e != cudaSuccess) return e;
     t1("k_big_cn");
   }
   if (ph & 2) {
     t0("k_big_cvs");
-    k_big_cvs<<<a.nw, kBigThreads, fixed, st>>>(a.walkers, a.coords, a.coff, a.step_off, a.step, a.log, a.ctr);
+    e = launch_chained(k_big_cvs, a.nw, kBigThreads, fixed, st, a.walkers, a.coords, a.coff, a.step_off, a.step, a.log,
+                       a.ctr, look ? 1 : 0);
+    if (e != cudaSuccess) return e;
     t1("k_big_cvs");
   }
   dim3 grid(a.nw, (a.max_stencil + kStencilPerBlock - 1) / kStencilPerBlock);
   if (ph & 4) {
     t0("k_big_deposit");
-    k_big_deposit<<<grid, kBigThreads, fixed, st>>>(a.walkers);
+    e = launch_chained(k_big_deposit, grid, kBigThreads, fixed, st, a.walkers);
+    if (e != cudaSuccess) return e;
     t1("k_big_deposit");
   }
   if ((ph & 8) && a.any_shared) {
     t0("k_big_refresh");
-    k_big_refresh<<<grid, kBigThreads, fixed, st>>>(a.walkers);
+    e = launch_chained(k_big_refresh, grid, kBigThreads, fixed, st, a.walkers);
+    if (e != cudaSuccess) return e;
     t1("k_big_refresh");
+  }
+  if ((ph & 16) && !look) {
+    t0("k_big_lookup");
+    e = launch_chained(k_big_lookup, a.nw, 32, fixed, st, a.walkers, a.step);
+    if (e != cudaSuccess) return e;
+    t1("k_big_lookup");
   }
   if (ph & 16) {
     t0("k_big_force");
-    k_big_force<<<dim3((a.max_atoms + kBigThreads - 1) / kBigThreads, a.nw), kBigThreads, fixed, st>>>(
-        a.walkers, a.forces, a.foff, a.force_step_off, a.mode, a.step);
+    const MdParams md = a.md ? *a.md : MdParams{};
+    e = launch_chained(k_big_force, dim3((a.max_atoms + kBigForceThreads - 1) / kBigForceThreads, a.nw),
+                       kBigForceThreads, 0, st, a.walkers, a.forces, a.foff, a.force_step_off, a.mode, a.step, md,
+                       a.md ? 1 : 0, a.xio, a.coff, a.traj, a.toff, a.traj_step_off);
+    if (e != cudaSuccess) return e;
     t1("k_big_force");
-  }
-  if ((ph & 16) && a.md) {
-    t0("k_big_move");
-    k_big_move<<<dim3((a.max_atoms + kBigThreads - 1) / kBigThreads, a.nw), kBigThreads, 0, st>>>(
-        a.walkers, *a.md, a.xio, a.coff, a.traj, a.toff, a.traj_step_off, a.step);
-    t1("k_big_move");
   }
   return cudaGetLastError();
 }
@@ -925,7 +963,7 @@ cudaError_t read_hill_heads(const WalkerDev *const *wd_host, int n, double *s3h,
 size_t big_cn_smem(const WalkerDev &hd) {
   int k = big_cn_index(hd);
   if (k < 0) return 0;
-  return (size_t)hd.cv[k].na * 16 + (size_t)(kBigThreads / 32) * hd.cv[k].na * 12;
+  return (size_t)hd.cv[k].na * 16 + (size_t)(kBigCnThreads / 32) * hd.cv[k].na * 12;
 }
 
 }  // namespace abp

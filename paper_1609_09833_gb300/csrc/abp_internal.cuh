@@ -95,6 +95,7 @@ struct WalkerDev {
   float kwall_f;
   void *fbuf;        // library-owned force records (abp_step -> abp_forces)
   void *jscratch;    // library-owned Jacobian scratch (plain form)
+  void *bpart;       // phased form: the partial sums of its coordination number's CTAs
   WalkerState *state;
   // a5 term tables of the closed-loop form, built at walker creation (or
   // null): per atom its count and kAtomTerms AtomTerm<Real> records, in CV

@@ -21,6 +21,23 @@ struct NvtxRange {
   NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// Launches a kernel that begins with chain_wait (abp_device.cuh): it may start
+// before the stream's previous kernel has ended.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // Optional per-kernel timing of a context (abp_ctx_tune ABP_TUNE_TIMING): the
 // launchers bracket each kernel launch with begin/end, which record CUDA
 // events on the launch's stream (read back by abp_kernel_times).
@@ -146,6 +163,7 @@ struct BigArgs {
   int max_stencil;           // largest stencil box (nodes) among the walkers
   int max_atoms;             // most atoms of a walker (the force phase's CTAs per walker)
   int any_shared;
+  int any_deposit;           // a walker of the call deposits at this step
   int phases;                // bits: 1 pairs, 2 CVs + heights, 4 deposit, 8 refresh, 16 forces (0 = all)
   LaunchTimer *timer;        // per-kernel timing (NULL: off)
   const MdParams *md;        // closed loop: the force phase also moves the atoms (NULL: open loop)
@@ -172,6 +190,7 @@ int md_group_bytes(const WalkerDev &hd, int fp64);
 cudaError_t launch_md(const MdRunArgs &a, int fp64, int dim, bool fast, cudaStream_t st);
 
 size_t big_scratch_bytes(const WalkerDev &hd);
+size_t big_part_bytes(const WalkerDev &hd);  // its coordination number's partial sums (bpart)
 // The force phase's per-atom term table of a phased-form walker (host side;
 // uploaded into its scratch): per atom, codes kind | k << 3 | position << 5
 // in the order a5 adds them. Returns -1 if an atom has more than kAtomTerms.
