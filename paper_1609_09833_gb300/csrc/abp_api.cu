@@ -1187,13 +1187,18 @@ static abp_status run_split(abp_ctx *ctx, const std::vector<abp_walker *> &ws, c
   return ABP_OK;
 }
 
-// Steps from which a batch of windowed-form walkers takes the split form: its
-// three launches cost ~25 us where the group form's one costs ~18 us and then
-// 0.2 us a step (well-tempered) or 1 us a step (mABP), each again per round of
-// walkers over the SMs. Measured, split / group, us: 64 walkers 32 steps 28 /
-// 23, 64 steps 31 / 31, 256 steps 50 / 66; 300 walkers 16 steps 27 / 37; mABP
-// 16 steps 27 / 29.
-int split_min_steps(int n, int sms, bool mabp) { return n > sms || mabp ? 16 : 64; }
+// Which form a call over windowed-form walkers takes (all give the same bits).
+// Short calls, one launch: measured against the group form, us, 64 walkers: 1
+// step 8.7 / 15.6, 32 steps 15.7 / 22.7; 700 walkers, 8 steps 32 / 76; its
+// mABP chain takes a hill at a time: 2 steps ~14 / 17, 4 steps 21 / 19. The
+// split form's three launches cost ~25 us where the group form's one costs
+// ~16 us and then 0.2 us a step (well-tempered) or 1 us a step (mABP), each
+// again per round of walkers over the SMs: 64 walkers 32 steps 28 / 23, 64
+// steps 31 / 31, 256 steps 50 / 66; 300 walkers 32 steps 31 / 44; mABP 16
+// steps 27 / 29.
+int short_max_steps(bool mabp) { return mabp ? 3 : 32; }
+int split_min_steps(int n, int sms, bool mabp) { return mabp ? 16 : n > sms ? 33 : 64; }
+constexpr int kShortSmem = 200 * 1024;  // shared memory of a short call's CTA, at most
 
 static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, const void *coords, int cdt,
                              const int64_t *coff, int64_t cstride, void *forces, const int64_t *foff,
@@ -1244,16 +1249,20 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     if (lw.empty()) continue;
     RunArgs a{};
     if ((st = sub_table(ctx, lw, li, &a.table))) return st;
-    // the split form (the same bits), unless a launch-shape knob asks for a
-    // group per walker or the call is too short for its three launches
-    bool mabp = true;
-    for (const abp_walker *w : lw) mabp = mabp && w->hd.method == ABP_METHOD_MABP;
-    bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1 &&
-                 (win ? nsteps >= split_min_steps((int)lw.size(), ctx->sms, mabp)
-                      : nsteps > 1 || (int)lw.size() > 2 * ctx->sms);
-    for (size_t i = 0; split && i < lw.size(); ++i) split = split_eligible(lw[i]->hd, win);
+    // unless a launch-shape knob asks for a group per walker (the same bits):
+    // short calls in one launch of the split form's parts, long ones in three
+    bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1;
+    bool mabp = false;
+    for (size_t i = 0; split && i < lw.size(); ++i) {
+      split = split_eligible(lw[i]->hd, win);
+      mabp = mabp || lw[i]->hd.method == ABP_METHOD_MABP;
+    }
     if (split) {
       SplitArgs s{};
+      s.table = a.table;
+      s.nw = (int)lw.size();
+      s.nsteps = nsteps;
+      s.last = 1;
       s.coords = coords;
       s.coff = reinterpret_cast<const long long *>(coff);
       s.cstride = cstride;
@@ -1264,9 +1273,21 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
       s.step0 = step0;
       s.log = ctx->log;
       s.ctr = ctx->ctr;
-      bool done = false;
-      if ((st = run_split(ctx, lw, a.table, win, s, nsteps, &done))) return st;
-      if (done) continue;
+      const int n = (int)lw.size();
+      if (win ? nsteps <= short_max_steps(mabp) : nsteps == 1 && n <= 2 * ctx->sms) {
+        int smem = 0;
+        for (const abp_walker *w : lw) smem = std::max(smem, short_smem(w->hd, win, nsteps));
+        if (smem <= kShortSmem) {
+          cudaError_t e = launch_short(s, win, smem, ctx->timer, ctx->stream);
+          if (e != cudaSuccess) return fail(ABP_ERR_CUDA, "short launch: %s", cudaGetErrorString(e));
+          continue;
+        }
+      }
+      if (!win || nsteps >= split_min_steps(n, ctx->sms, mabp)) {
+        bool done = false;
+        if ((st = run_split(ctx, lw, a.table, win, s, nsteps, &done))) return st;
+        if (done) continue;
+      }
     }
     if ((st = pick_shape(ctx, lw.data(), (int)lw.size(), fp64, nsteps, win, &a.G, &a.groups_per_cta,
                          &a.group_bytes, &a.tile_budget)))

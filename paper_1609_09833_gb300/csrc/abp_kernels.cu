@@ -1287,6 +1287,7 @@ __global__ void __launch_bounds__(256) k_deliver(const TableEntry *table, int nw
   const TableEntry te = table[blockIdx.x];
   const WalkerDev *wd = te.wd;
   const int natoms = wd->natoms;
+  chain_wait();
   const R4 *src = reinterpret_cast<const R4 *>(wd->fbuf);
   R4 *dst = reinterpret_cast<R4 *>(forces) + foff[te.idx];
   for (int i = threadIdx.x; i < natoms; i += blockDim.x) store_force<Real>(dst + i, src[i], mode);
@@ -1295,11 +1296,8 @@ __global__ void __launch_bounds__(256) k_deliver(const TableEntry *table, int nw
 cudaError_t launch_deliver(const TableEntry *table, int nw, void *forces, const long long *foff, int mode, int fp64,
                            cudaStream_t st) {
   if (nw == 0) return cudaSuccess;
-  if (fp64)
-    k_deliver<double><<<nw, 128, 0, st>>>(table, nw, forces, foff, mode);
-  else
-    k_deliver<float><<<nw, 128, 0, st>>>(table, nw, forces, foff, mode);
-  return cudaGetLastError();
+  if (fp64) return launch_chained(k_deliver<double>, nw, 128, 0, st, table, nw, forces, foff, mode);
+  return launch_chained(k_deliver<float>, nw, 128, 0, st, table, nw, forces, foff, mode);
 }
 
 // ---------------------------------------------------------------- abp_bias_readout

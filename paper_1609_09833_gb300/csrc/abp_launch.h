@@ -118,6 +118,9 @@ void split_shape(const WalkerDev &hd, bool win, SplitShape *s);
 size_t split_step_bytes();
 int split_jac_records(const WalkerDev &hd);
 int split_term_words(const WalkerDev &hd);
+// Short calls: dynamic shared bytes of a walker, and the one launch.
+int short_smem(const WalkerDev &hd, bool win, int nsteps);
+cudaError_t launch_short(const SplitArgs &a, bool win, int smem, LaunchTimer *tm, cudaStream_t st);
 cudaError_t launch_split(const SplitArgs &a, const SplitShape &s, int sms, LaunchTimer *tm, cudaStream_t st);
 
 struct PlainArgs {

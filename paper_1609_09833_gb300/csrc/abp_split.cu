@@ -41,7 +41,8 @@ namespace {
 
 using Step = StepRec<float>;
 constexpr int kStepWords = (int)(sizeof(Step) / 4);
-constexpr int kCvThreads = 128, kCnThreads = 128, kChainThreads = 512, kHistThreads = 128, kForceThreads = 128;
+constexpr int kCvThreads = 128, kCnThreads = 128, kChainThreads = 512, kHistThreads = 128, kForceThreads = 128,
+              kShortThreads = 256, kOneThreads = (4 + 2) * 32;
 constexpr int kHistWin = 64;  // most mABP hills applied to a node between its load and its store
 
 __host__ __device__ constexpr int fixed_bytes_f() { return (int)((sizeof(GroupFixed<float>) + 31) & ~(size_t)31); }
@@ -118,6 +119,48 @@ __host__ __device__ inline CvLayout cv_layout(int natoms, const CvDev *cv, int d
   return L;
 }
 
+// The step records of nt steps whose coordinates are on their way to xs (rows
+// of xst records) and whose lists are being staged: one lane per (CV, step),
+// two for a COM distance, the finiteness of every atom, the flags.
+__device__ __forceinline__ void window_records(const Grp &g, GroupFixed<float> *fx, const float4 *xs, int xst, Step *st,
+                                               int nt, long long s0, DevCounters *ctr) {
+  const WalkerDev &wd = fx->wd;
+  const int d = wd.g.d, natoms = wd.natoms;
+  if (g.t == 0) fx->winbad[0] = 0;
+  cp_async_wait_all();
+  __syncthreads();
+  // tasks: whole warps per CV; warps go round the task list
+  int base[kMaxCv + 1];
+  base[0] = 0;
+  for (int k = 0; k < d; ++k) base[k + 1] = base[k] + align32((wd.cv[k].type == ABP_CV_COM_DIST ? 2 : 1) * nt);
+  for (int task = g.t; task < base[d]; task += g.G) {
+    int k = 0;
+    while (k + 1 < d && task >= base[k + 1]) ++k;
+    const int r = task - base[k];
+    if (wd.cv[k].type == ABP_CV_COM_DIST) {
+      const int j = min(r >> 1, nt - 1);
+      window_com2<float>(fx, xs + j * xst, k, (s0 + j) % wd.stride == 0, (r >> 1) < nt, r & 1, st[j]);
+    } else if (r < nt) {
+      window_cv<float>(fx, xs + r * xst, k, (s0 + r) % wd.stride == 0, st[r]);
+    }
+  }
+  unsigned mine = 0;
+  for (Iter2 it(g.t, g.G, natoms); it.j < nt; it.next())
+    if (!finite_rec<float>(xs[it.j * xst + it.i])) mine |= 1u << it.j;
+  mine = __reduce_or_sync(0xffffffffu, mine);
+  if (g.lane == 0 && mine) atomicOr(&fx->winbad[0], mine);
+  __syncthreads();
+  const unsigned bad = fx->winbad[0];
+  if (g.t == 0 && bad) atomicAdd(&ctr->nonfinite, __popc(bad));
+  for (int j = g.t; j < nt; j += g.G) {
+    if ((bad >> j) & 1)
+      st[j].flags = ABP_WFLAG_NONFINITE;
+    else
+      step_flags<float>(d, (s0 + j) % wd.stride == 0, st[j]);
+  }
+  __syncthreads();
+}
+
 // One window (W steps, as window_steps gives for the walker) of one walker:
 // its coordinates into shared memory, one lane per (CV, step) -- two for a
 // COM distance --, the finiteness of every atom on the threads left over,
@@ -141,40 +184,7 @@ __global__ void __launch_bounds__(kCvThreads) k_sp_cv(SplitArgs a) {
     cp_async16(xs + it.j * L.xst + it.i, cin + (long long)it.j * a.cstride + it.i);
   cp_async_commit();
   stage_lists(g, wd, smem + L.lists, fx->ia, fx->ib, fx->wa, fx->wb);
-  if (g.t == 0) fx->winbad[0] = 0;
-  cp_async_wait_all();
-  __syncthreads();
-  const long long s0 = a.step0 + a.t0 + t0;
-  // tasks: whole warps per CV; warps go round the task list
-  int base[kMaxCv + 1];
-  base[0] = 0;
-  for (int k = 0; k < d; ++k) base[k + 1] = base[k] + align32((wd.cv[k].type == ABP_CV_COM_DIST ? 2 : 1) * nt);
-  for (int task = g.t; task < base[d]; task += g.G) {
-    int k = 0;
-    while (k + 1 < d && task >= base[k + 1]) ++k;
-    const int r = task - base[k];
-    if (wd.cv[k].type == ABP_CV_COM_DIST) {
-      const int j = min(r >> 1, nt - 1);
-      window_com2<float>(fx, xs + j * L.xst, k, (s0 + j) % wd.stride == 0, (r >> 1) < nt, r & 1, st[j]);
-    } else if (r < nt) {
-      window_cv<float>(fx, xs + r * L.xst, k, (s0 + r) % wd.stride == 0, st[r]);
-    }
-  }
-  unsigned mine = 0;
-  for (Iter2 it(g.t, g.G, natoms); it.j < nt; it.next())
-    if (!finite_rec<float>(xs[it.j * L.xst + it.i])) mine |= 1u << it.j;
-  mine = __reduce_or_sync(0xffffffffu, mine);
-  if (g.lane == 0 && mine) atomicOr(&fx->winbad[0], mine);
-  __syncthreads();
-  const unsigned bad = fx->winbad[0];
-  if (g.t == 0 && bad) atomicAdd(&a.ctr->nonfinite, __popc(bad));
-  for (int j = g.t; j < nt; j += g.G) {
-    if ((bad >> j) & 1)
-      st[j].flags = ABP_WFLAG_NONFINITE;
-    else
-      step_flags<float>(d, (s0 + j) % wd.stride == 0, st[j]);
-  }
-  __syncthreads();
+  window_records(g, fx, xs, L.xst, st, nt, a.step0 + a.t0 + t0, a.ctr);
   load_words(g, walker_steps_of(a, blockIdx.x) + t0, st, nt * kStepWords);
 }
 
@@ -450,6 +460,13 @@ __device__ __forceinline__ void step_lookup(const WalkerDev &wd, Step *sp) {
 #pragma unroll
     for (int q = 0; q <= DIM; ++q) acc[q] = fma_rn(wc, v[q], acc[q]);
   }
+  if (wd.method == ABP_METHOD_MABP) {  // the nearest node's histograms
+    float V, dvm[3] = {0.f, 0.f, 0.f};
+    mabp_bias<float>(wd, acc, V, dvm);
+    acc[0] = V;
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) acc[1 + k] = dvm[k];
+  }
   sp->V = acc[0];
 #pragma unroll
   for (int k = 0; k < DIM; ++k)
@@ -492,7 +509,7 @@ __device__ __forceinline__ void chain_height(const Grp &g, GroupFixed<float> *fx
                                              const DepositLog &log) {
   const GridDev &gd = fx->wd.g;
   double term = 0;
-  if (g.lane < (1 << DIM)) {
+  if (g.lane < (1 << DIM) && fx->wd.method != ABP_METHOD_MABP) {  // mABP hills: fixed height
     double w = 1;
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
@@ -547,6 +564,15 @@ __device__ __forceinline__ void chain_body(const Grp &g, GroupFixed<float> *fx, 
   }
 }
 
+__device__ __forceinline__ void chain_any(const Grp &g, GroupFixed<float> *fx, Step *st, const SplitArgs &a) {
+  if (fx->wd.g.d == 1)
+    chain_body<1>(g, fx, st, a);
+  else if (fx->wd.g.d == 2)
+    chain_body<2>(g, fx, st, a);
+  else
+    chain_body<3>(g, fx, st, a);
+}
+
 // One CTA per walker. Bound by the chain of deposits: two rounds of grid
 // reads (the height's corners, the stencil) and their barriers each.
 __global__ void __launch_bounds__(kChainThreads, 1) k_sp_chain(SplitArgs a) {
@@ -560,12 +586,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_sp_chain(SplitArgs a) {
   if (a.terms && a.t0 == 0) 
     list_atom_terms(g, wd, atom_terms_of(a, blockIdx.x), atom_counts_of(a, blockIdx.x, wd.natoms));
   Step *st = walker_steps_of(a, blockIdx.x);
-  if (wd.g.d == 1)
-    chain_body<1>(g, fx, st, a);
-  else if (wd.g.d == 2)
-    chain_body<2>(g, fx, st, a);
-  else
-    chain_body<3>(g, fx, st, a);
+  chain_any(g, fx, st, a);
   g.sync();
   if (a.last && g.t == 0) state_out(wd, st[a.nsteps - 1], a.step0 + a.t0 + a.nsteps - 1);
 }
@@ -1019,6 +1040,227 @@ __global__ void __launch_bounds__(kCnfThreads) k_sp_cnf(SplitArgs a) {
   }
 }
 
+// ---------------------------------------------------------------- short calls
+//
+// The same parts in one launch, one CTA per walker, for calls of a few steps
+// (a host engine's one step per call): records and Jacobians stay in shared
+// memory. Bound by latency: the descriptor, the lists and coordinates, the
+// CVs, the grid's corners, one after the other. Descriptors and lists are read
+// before the earlier work of the stream is waited for. One step of one walker
+// of two 16-atom groups and a dihedral: 16.2 us with a group of the windowed
+// form, 8.2 us here; of 16 pocket walkers of 40 x 400 pairs 22.6 -> 14.6 us.
+
+// Up to kWinMax steps of a walker of k_sp_cv's kind.
+__global__ void __launch_bounds__(kShortThreads) k_sp_short(SplitArgs a) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  const Grp g = cta_grp();
+  GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
+  const TableEntry te = a.table[blockIdx.x];
+  load_words(g, &fx->wd, te.wd, (int)(sizeof(WalkerDev) / 4));
+  g.sync();
+  const WalkerDev &wd = fx->wd;
+  const int natoms = wd.natoms, d = wd.g.d, nt = a.nsteps;
+  const CvLayout L = cv_layout(natoms, wd.cv, d, nt);
+  Step *st = reinterpret_cast<Step *>(smem + L.recs);
+  float4 *xs = reinterpret_cast<float4 *>(smem + L.xs);
+  stage_lists(g, wd, smem + L.lists, fx->ia, fx->ib, fx->wa, fx->wb);
+  // this thread's atom's a5 terms
+  const AtomTerm<float> *terms = reinterpret_cast<const AtomTerm<float> *>(wd.aterms);
+  const int ne0 = g.t < natoms ? wd.acnt[g.t] : 0;
+  AtomTerm<float> mine[kAtomTerms];
+#pragma unroll
+  for (int q = 0; q < kAtomTerms; ++q)
+    mine[q] = q < ne0 ? terms[(size_t)g.t * kAtomTerms + q] : AtomTerm<float>{0.f, 0};
+  chain_wait();
+  const float4 *cin = reinterpret_cast<const float4 *>(a.coords) + a.coff[te.idx];
+  for (Iter2 it(g.t, g.G, natoms); it.j < nt; it.next())
+    cp_async16(xs + it.j * L.xst + it.i, cin + (long long)it.j * a.cstride + it.i);
+  cp_async_commit();
+  window_records(g, fx, xs, L.xst, st, nt, a.step0, a.ctr);
+  chain_any(g, fx, st, a);
+  g.sync();
+  if (g.t == 0) state_out(wd, st[nt - 1], a.step0 + nt - 1);
+  for (int i = g.t; i < nt * kMaxCv * 12; i += g.G) {
+    const int j = i / (kMaxCv * 12), q = i - j * (kMaxCv * 12), k = q / 12;
+    float *v = &st[j].jac[0][0] + q;
+    if (k < d) *v = __fmul_rn(*v, st[j].dv[k]);
+  }
+  g.sync();
+  const int mode = a.forces ? a.mode : ABP_FORCES_OVERWRITE;
+  for (int at = g.t; at < natoms; at += g.G) {
+    int ne = ne0;
+    if (at != g.t) {
+      ne = wd.acnt[at];
+#pragma unroll
+      for (int q = 0; q < kAtomTerms; ++q)
+        mine[q] = q < ne ? terms[(size_t)at * kAtomTerms + q] : AtomTerm<float>{0.f, 0};
+    }
+    for (int j = 0; j < nt; ++j) {
+      float4 *fo = force_out(a, wd, te.idx, j);
+      if (!fo) continue;
+      if (st[j].flags & ABP_WFLAG_NONFINITE) {
+        if (mode == ABP_FORCES_OVERWRITE) fo[at] = make_float4(0.f, 0.f, 0.f, 0.f);
+        continue;
+      }
+      float f0 = 0.f, f1 = 0.f, f2 = 0.f;
+#pragma unroll
+      for (int q = 0; q < kAtomTerms; ++q)
+        if (q < ne) {
+          const float *v = &st[j].jac[0][0] + mine[q].off;
+          f0 = fma_rn(mine[q].w, v[0], f0);
+          f1 = fma_rn(mine[q].w, v[1], f1);
+          f2 = fma_rn(mine[q].w, v[2], f2);
+        }
+      store_force<float>(fo + at, make_float4(f0, f1, f2, 0.f), mode);
+    }
+  }
+}
+
+// Shared memory of k_sp_one: GroupFixed | step record | lists | A gradients |
+// coordinates | gradient records | forces.
+struct OneLayout {
+  int rec, lists, lig, xs, jac, fs, total;
+};
+__host__ __device__ inline OneLayout one_layout(int natoms, const CvDev *cv, int d) {
+  OneLayout L;
+  L.rec = fixed_bytes_f();
+  L.lists = up32(L.rec + (int)sizeof(Step));
+  L.lig = L.lists + list_bytes(cv, d);
+  L.xs = up32(L.lig + kCnWarps * cn_lig_floats(cv, d) * 4);
+  L.jac = L.xs + natoms * 16;
+  L.fs = L.jac + cn_records(cv, d) * 16;
+  L.total = L.fs + natoms * 16;
+  return L;
+}
+
+// One step of a walker of k_sp_cn's kind: the coordination numbers on the
+// first four warps, COM distances on the fifth, dihedrals on the sixth.
+__global__ void __launch_bounds__(kOneThreads) k_sp_one(SplitArgs a) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  __shared__ float red[kCnWarps][2];
+  const Grp g = cta_grp();
+  GroupFixed<float> *fx = reinterpret_cast<GroupFixed<float> *>(smem);
+  const TableEntry te = a.table[blockIdx.x];
+  load_words(g, &fx->wd, te.wd, (int)(sizeof(WalkerDev) / 4));
+  g.sync();
+  const WalkerDev &wd = fx->wd;
+  const int natoms = wd.natoms, d = wd.g.d;
+  const OneLayout L = one_layout(natoms, wd.cv, d);
+  Step *st = reinterpret_cast<Step *>(smem + L.rec);
+  float *ligs = reinterpret_cast<float *>(smem + L.lig);
+  float4 *x = reinterpret_cast<float4 *>(smem + L.xs), *J = reinterpret_cast<float4 *>(smem + L.jac);
+  float4 *fs = reinterpret_cast<float4 *>(smem + L.fs);
+  stage_lists(g, wd, smem + L.lists, fx->ia, fx->ib, fx->wa, fx->wb);
+  for (int i = g.t; i < natoms; i += g.G) fs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  chain_wait();
+  const float4 *cin = reinterpret_cast<const float4 *>(a.coords) + a.coff[te.idx];
+  for (int i = g.t; i < natoms; i += g.G) cp_async16(x + i, cin + i);
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
+  float4 *fo = force_out(a, wd, te.idx, 0);
+  const int mode = a.forces ? a.mode : ABP_FORCES_OVERWRITE;
+  if (__syncthreads_or(!step_finite(x, natoms, g.t, g.G))) {
+    if (mode == ABP_FORCES_OVERWRITE)
+      for (int i = g.t; i < natoms; i += g.G) fo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (g.t == 0) {
+      wd.state->flags = ABP_WFLAG_NONFINITE;
+      atomicAdd(&a.ctr->nonfinite, 1);
+    }
+    return;
+  }
+  const bool dep = a.step0 % wd.stride == 0;
+  float4 *Jk = J;
+  for (int k = 0; k < d; ++k) {
+    const CvDev &c = wd.cv[k];
+    if (c.type == ABP_CV_COM_DIST) {
+      if (g.warp == kCnWarps) {
+        float s = 0.f, sl = 0.f;
+        const int fl = com_one_warp(c, fx->ia[k], fx->ib[k], fx->wa[k], fx->wb[k], x, g.lane, s, sl, st->jac[k]);
+        if (g.lane == 0) window_cv_rec<float>(wd, k, s, sl, fl, dep, *st);
+      }
+    } else if (c.type == ABP_CV_DIHEDRAL) {
+      if (g.t == g.G - 1) window_cv<float>(fx, x, k, dep, *st);
+    } else {
+      const float c6 = -6.f * (float)c.inv_r0sq;
+      if (g.warp < kCnWarps) {
+        float h[1], l[1];
+        cn_warp_any(c, fx->ia[k], fx->ib[k], x, Jk + c.na, ligs + g.warp * c.na * 3, false, g.lane, 8 * g.warp,
+                    8 * kCnWarps, h[0], l[0]);
+        warp_sum_ff<1>(h, l);
+        if (g.lane == 0) {
+          red[g.warp][0] = h[0];
+          red[g.warp][1] = l[0];
+        }
+      }
+      __syncthreads();
+      if (g.t == 0) {
+        float sh = red[0][0], sl = red[0][1];
+#pragma unroll
+        for (int v = 1; v < kCnWarps; ++v) ff_add<float>(sh, sl, red[v][0], red[v][1]);
+        window_cv_rec<float>(wd, k, sh, sl, 0, dep, *st);
+      }
+      for (int i = g.t; i < c.na; i += g.G) {
+        float s3[3];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          s3[e] = ligs[3 * i + e];
+#pragma unroll
+          for (int v = 1; v < kCnWarps; ++v) s3[e] = __fadd_rn(s3[e], ligs[(v * c.na + i) * 3 + e]);
+        }
+        Jk[i] = make_float4(__fmul_rn(c6, s3[0]), __fmul_rn(c6, s3[1]), __fmul_rn(c6, s3[2]), 0.f);
+      }
+      __syncthreads();  // the scratch is free again
+      Jk += c.na + c.nb;
+    }
+  }
+  __syncthreads();
+  if (g.t == 0) step_flags<float>(d, dep, *st);
+  __syncthreads();
+  chain_any(g, fx, st, a);
+  g.sync();
+  if (g.t == 0) state_out(wd, *st, a.step0);
+  // a5: list by list (an atom appears at most once in a list), CV by CV
+  int jpos = 0;
+  for (int k = 0; k < d; ++k) {
+    const CvDev &c = wd.cv[k];
+    const bool com = c.type == ABP_CV_COM_DIST, cn = c.type == ABP_CV_COORD;
+    const float dv = st->dv[k];
+    const float u0 = __fmul_rn(st->jac[k][0], dv), u1 = __fmul_rn(st->jac[k][1], dv), u2 = __fmul_rn(st->jac[k][2], dv);
+    for (int lst = 0; lst < (com || cn ? 2 : 1); ++lst) {
+      const int n = lst ? c.nb : (com || cn ? c.na : 4);
+      const int32_t *list = lst ? fx->ib[k] : fx->ia[k];
+      for (int i = g.t; i < n; i += g.G) {
+        float w, v0, v1, v2;
+        if (com) {
+          w = lst ? -fx->wb[k][i] : fx->wa[k][i];
+          v0 = u0;
+          v1 = u1;
+          v2 = u2;
+        } else if (cn) {
+          const float4 j = J[jpos + (lst ? c.na : 0) + i];
+          w = -dv;
+          v0 = j.x;
+          v1 = j.y;
+          v2 = j.z;
+        } else {
+          w = -dv;
+          v0 = st->jac[k][3 * i];
+          v1 = st->jac[k][3 * i + 1];
+          v2 = st->jac[k][3 * i + 2];
+        }
+        float4 &f = fs[list[i]];
+        f.x = fma_rn(w, v0, f.x);
+        f.y = fma_rn(w, v1, f.y);
+        f.z = fma_rn(w, v2, f.z);
+      }
+      __syncthreads();
+    }
+    if (cn) jpos += c.na + c.nb;
+  }
+  for (int i = g.t; i < natoms; i += g.G) store_force<float>(fo + i, fs[i], mode);
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- host side
@@ -1052,6 +1294,22 @@ void split_shape(const WalkerDev &hd, bool win, SplitShape *s) {
     s->wt += 1;
   s->min_dim = s->min_dim == 0 ? hd.g.d : min(s->min_dim, hd.g.d);
   s->max_atoms = max(s->max_atoms, hd.natoms);
+}
+
+int short_smem(const WalkerDev &hd, bool win, int nsteps) {
+  return win ? cv_layout(hd.natoms, hd.cv, hd.g.d, nsteps).total : one_layout(hd.natoms, hd.cv, hd.g.d).total;
+}
+
+cudaError_t launch_short(const SplitArgs &a, bool win, int smem, LaunchTimer *tm, cudaStream_t st) {
+  void (*k)(SplitArgs) = win ? k_sp_short : k_sp_one;
+  const char *name = win ? "k_sp_short" : "k_sp_one";
+  cudaError_t e = smem_attr(reinterpret_cast<const void *>(k), smem);
+  if (e != cudaSuccess) return e;
+  NvtxRange nv(name);
+  if (tm) tm->begin(name, st);
+  e = launch_chained(k, a.nw, win ? kShortThreads : kOneThreads, smem, st, a);
+  if (tm) tm->end(name, st);
+  return e;
 }
 
 cudaError_t launch_split(const SplitArgs &a0, const SplitShape &s, int sms, LaunchTimer *tm, cudaStream_t st) {
