@@ -189,12 +189,15 @@ struct abp_walker {
   // most 64 atoms of at most two a5 terms each, COM groups of at most 16
   // atoms, the other CVs dihedrals
   bool md_fast = false;
+  bool md_line = false;  // FP64, well-tempered, one COM distance: k_md_line takes it
   long long cost = 0;  // rough work estimate used to order batched launches
 };
 
 namespace {
 
 constexpr size_t kPoolKeep = 256u << 20;     // bytes the scratch pool of a device keeps between calls
+constexpr size_t kNoiseScratch = 64u << 20;  // noise of a block of closed-loop steps
+constexpr int kLineMaxAtoms = 2048;          // atoms of a walker of k_md_line (its coordinates fit shared memory)
 constexpr size_t kReadoutChunk = 32u << 20;  // staging bytes of a readout
 
 // The library's memory pool of a device, shared by its contexts there: made
@@ -932,6 +935,7 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
     void *pc = nullptr, *pt = nullptr;
     if (fp64) {
       std::vector<AtomTerm<double>> tt;
+      w->md_line = ncv == 1 && d->cv[0].type == ABP_CV_COM_DIST && !mabp && d->natoms <= kLineMaxAtoms;
       atom_term_tables<double>(d, ncv, tcnt, tt);
       st = upload(w, tt.data(), tt.size() * sizeof(AtomTerm<double>), &pt);
     } else {
@@ -1462,6 +1466,32 @@ abp_status abp_md_run(abp_ctx *ctx, abp_walker *const *walkers, int n, void *coo
     a.tstride = traj_step_stride;
     bool fast = !fp64;
     for (abp_walker *w : lw) fast = fast && w->md_fast;
+    // FP64 walkers of one COM distance, one an SM at most (more of them fill
+    // the FP64 pipes as it is), in blocks of steps whose noise fits the scratch
+    bool line = fp64 && dim == 1 && (int)lw.size() <= ctx->sms;
+    int max_atoms = 1;
+    for (abp_walker *w : lw) {
+      line = line && w->md_line;
+      max_atoms = std::max(max_atoms, w->hd.natoms);
+    }
+    if (line) {
+      const size_t per_step = md_noise_bytes(a.r.nw, max_atoms, 1);
+      const int block = (int)std::min<size_t>(nsteps, std::max<size_t>(1, kNoiseScratch / per_step));
+      Scratch noise(ctx, per_step * block);
+      if (noise.p) {
+        const long long fstep = force_step_stride * (long long)(fp64 ? 32 : 16), tstep = traj_step_stride * 32ll;
+        for (int t = 0; t < nsteps; t += block) {
+          MdRunArgs b = a;
+          b.r.step0 = step0 + t;
+          b.r.nsteps = std::min(block, nsteps - t);
+          if (forces_dev) b.r.forces = static_cast<unsigned char *>(forces_dev) + t * fstep;
+          if (traj_dev) b.traj = static_cast<unsigned char *>(traj_dev) + t * tstep;
+          cudaError_t e = launch_md_line(b, max_atoms, noise.p, ctx->timer, ctx->stream);
+          if (e != cudaSuccess) return fail(ABP_ERR_CUDA, "closed-loop launch: %s", cudaGetErrorString(e));
+        }
+        continue;
+      }
+    }
     NvtxRange nv("k_md");
     if (ctx->timer) ctx->timer->begin("k_md", ctx->stream);
     cudaError_t e = launch_md(a, fp64, dim, fast, ctx->stream);

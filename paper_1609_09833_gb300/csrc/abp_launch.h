@@ -191,6 +191,10 @@ struct MdRunArgs {
 // Closed-loop form of walkers whose CVs a thread evaluates (abp_md.cu).
 int md_group_bytes(const WalkerDev &hd, int fp64);
 cudaError_t launch_md(const MdRunArgs &a, int fp64, int dim, bool fast, cudaStream_t st);
+// Closed-loop form of FP64 walkers of one COM distance, with the noise of its
+// steps in `noise` (md_noise_bytes).
+size_t md_noise_bytes(int nw, int max_atoms, int nsteps);
+cudaError_t launch_md_line(const MdRunArgs &a, int max_atoms, void *noise, LaunchTimer *tm, cudaStream_t st);
 
 size_t big_scratch_bytes(const WalkerDev &hd);
 size_t big_part_bytes(const WalkerDev &hd);  // its coordination number's partial sums (bpart)

@@ -721,11 +721,322 @@ __global__ void __launch_bounds__(256, 1) k_md(MdRunArgs a) {
   }
 }
 
+// ---------------------------------------------------------------- FP64, one COM distance
+//
+// An FP64 instruction of a warp takes 64 cycles of its SM quarter on this part,
+// dependent or not (measured), so a step costs the FP64 instructions the busiest
+// warp issues. This form of the closed loop, for FP64 well-tempered walkers whose
+// one CV is a COM distance, spreads them: coordinate q of every atom belongs to
+// warp q (its sums, its force, its move, with no barrier between a move and the
+// next step's sums); behind the first barrier warp 0 forms the distance, the axis
+// state and the look-up, warp 1 the distance again and the unit separation, warp
+// 2 the distance and the CV potential's gradient; the noise comes from a kernel
+// of its own on the other SMs (k_md_noise), scaled and read a step ahead. About
+// 40 FP64 instructions a step on the busiest warp against ~130 in k_md: one
+// walker of two 8-atom groups, 4.30 -> 2.3 us per step. The same
+// operations in the same order as k_md, so the same bits.
+
+// The noise of steps [0, nsteps) of a block, c2 xi, as [walker][step][coordinate][atom].
+__global__ void __launch_bounds__(128) k_md_noise(const TableEntry *table, MdParams md, long long step0, int nsteps,
+                                                  int stride, double *out) {
+  const TableEntry te = table[blockIdx.y];
+  const int natoms = te.wd->natoms;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)nsteps * natoms) return;
+  const int t = (int)(i / natoms), at = (int)(i - (long long)t * natoms);
+  double n[3];
+  md_normals(md.seed, te.stream, step0 + t, at, n);
+  double *p = out + ((size_t)blockIdx.y * nsteps + t) * stride + at;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) p[q * natoms] = mul_rn(md.c2, n[q]);
+}
+
+constexpr int kLineThreads = 128;
+
+// Shared memory of k_md_line: GroupFixed | step record | coordinates [3][natoms] and pad.
+struct LineLayout {
+  int st, xs, total;
+};
+__host__ __device__ inline LineLayout line_layout(int natoms) {
+  LineLayout L;
+  L.st = md_fixed_bytes<double>();
+  L.xs = L.st + align32((int)sizeof(StepRec<double>));
+  L.total = align32(L.xs + 4 * natoms * 8);
+  return L;
+}
+
+// The same value, which the compiler may not compute with ahead of this point:
+// keeps one warp's FP64 work out of the others' instruction streams.
+__device__ __forceinline__ double here(double x) {
+  asm volatile("" : "+d"(x));
+  return x;
+}
+
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+__global__ void __launch_bounds__(kLineThreads) k_md_line(MdRunArgs a, const double *noise, int nstride) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  __shared__ double ds[3], us[3], dUs, dvs;
+  __shared__ int bads[4], sing;
+  const RunArgs &ra = a.r;
+  const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;  // q < 3: this warp's coordinate
+  Grp g;
+  g.G = kLineThreads;
+  g.gid = 0;
+  g.t = tid;
+  g.lane = lane;
+  g.warp = q;
+  g.nwarps = kLineThreads / 32;
+  GroupFixed<double> *fx = reinterpret_cast<GroupFixed<double> *>(smem);
+  const TableEntry te = ra.table[blockIdx.x];
+  {
+    const int *s = reinterpret_cast<const int *>(te.wd);
+    int *d = reinterpret_cast<int *>(&fx->wd);
+    for (int i = tid; i < (int)(sizeof(WalkerDev) / 4); i += kLineThreads) d[i] = s[i];
+  }
+  __syncthreads();
+  const WalkerDev &wd = fx->wd;
+  const CvDev &c = wd.cv[0];
+  const GridDev &gd = wd.g;
+  const int natoms = wd.natoms;
+  const LineLayout L = line_layout(natoms);
+  StepRec<double> &st = *reinterpret_cast<StepRec<double> *>(smem + L.st);
+  double *xs = reinterpret_cast<double *>(smem + L.xs);  // [4][natoms]: x, y, z, the records' pad
+  D4 *cio = reinterpret_cast<D4 *>(const_cast<void *>(ra.coords)) + ra.coff[te.idx];
+  for (int i = tid; i < natoms; i += kLineThreads) {
+    const D4 p = cio[i];
+    xs[i] = p.x;
+    xs[natoms + i] = p.y;
+    xs[2 * natoms + i] = p.z;
+    xs[3 * natoms + i] = p.w;
+  }
+  __syncthreads();
+  double *x = xs + (q < 3 ? q : 0) * natoms;
+  // this lane's first atom of its group's sum (group A on lanes 0-15, B on 16-31)
+  const bool gb = lane >= 16;
+  const int32_t *list = gb ? c.ib : c.ia;
+  const double *wts = gb ? c.wb64 : c.wa64;
+  const int ng = gb ? c.nb : c.na, first = list[0], mine = (lane & 15) < ng ? list[lane & 15] : -1;
+  const double wmine = mine >= 0 ? wts[lane & 15] : 0.0;
+  // the first atom of this lane's moves: its a5 terms
+  const AtomTerm<double> *terms = reinterpret_cast<const AtomTerm<double> *>(wd.aterms);
+  const int ne0 = lane < natoms ? wd.acnt[lane] : 0;
+  const double w00 = ne0 > 0 ? terms[lane * kAtomTerms].w : 0.0, w01 = ne0 > 1 ? terms[lane * kAtomTerms + 1].w : 0.0;
+  const MdCoef<double> mc = md_coef<double>(a.md);
+  const double invD = gd.invD[0], u0 = gd.u0[0];
+  const int n0 = gd.n[0], per = gd.periodic[0];
+  const bool wall = wd.kwall > 0;
+  const unsigned char *rec = reinterpret_cast<const unsigned char *>(gd.rec);
+  D4 *fout = ra.forces ? reinterpret_cast<D4 *>(ra.forces) + ra.foff[te.idx] : reinterpret_cast<D4 *>(wd.fbuf);
+  const int fmode = ra.forces ? ra.mode : ABP_FORCES_OVERWRITE;
+  D4 *tout = a.traj ? reinterpret_cast<D4 *>(a.traj) + a.toff[te.idx] : nullptr;
+  const double *nz = noise + (size_t)blockIdx.x * ra.nsteps * nstride + (q < 3 ? q : 0) * natoms;
+  const long long step0 = ra.step0;
+  const long long rem = step0 % wd.stride;
+  long long next_dep = rem == 0 ? 0 : wd.stride - rem;
+  if (q < 3) {
+    int bad = 0;
+    for (int i = lane; i < natoms; i += 32) bad |= finite_bits(x[i]) ? 0 : 1;
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) bads[q] = bad;
+  }
+  int last = -1, flags = 0;
+  bool stopped = false;
+  double V = 0, s_last = 0;
+  double nnext = q < 3 && lane < natoms && ra.nsteps > 0 ? nz[lane] : 0.0;
+  for (int t = 0; t < ra.nsteps; ++t) {
+    const bool dep = t == next_dep;
+    if (dep) next_dep += wd.stride;
+    const double noise0 = nnext;
+    if (q < 3 && lane < natoms && t + 1 < ra.nsteps) nnext = nz[(size_t)(t + 1) * nstride + lane];
+    // a1, coordinate q: the groups' weighted offsets from their first atoms (com_warp)
+    if (q < 3) {
+      const double p0 = x[first];
+      double h = 0;
+      if (mine >= 0) h = fma_rn(wmine, sub_rn(x[mine], p0), h);
+      for (int i = (lane & 15) + 16; i < ng; i += 16) h = fma_rn(wts[i], sub_rn(x[list[i]], p0), h);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) h = add_rn(h, __shfl_xor_sync(0xffffffffu, h, o));
+      const double hb = __shfl_sync(0xffffffffu, h, 16), pb = __shfl_sync(0xffffffffu, p0, 16);
+      if (lane == 0) {
+        double d = add_rn(sub_rn(pb, p0), sub_rn(hb, h));
+        if (c.pbc) d = min_image<double, true>(d, c.box[q], c.inv_box[q]);
+        ds[q] = d;
+      }
+    }
+    // (reconverge after every one-lane region: a warp that meets the barrier in
+    // two parts runs what follows, and its FP64 instructions, twice)
+    __syncwarp();
+    __syncthreads();
+    if (bads[0] | bads[1] | bads[2]) {
+      // this walker stops here: its state says so, its atoms stay
+      if (tid == 0) {
+        wd.state->flags = ABP_WFLAG_NONFINITE;
+        atomicAdd(&ra.ctr->nonfinite, 1);
+      }
+      stopped = true;
+      break;
+    }
+    const double d0 = ds[0], d1 = ds[1], d2 = ds[2];
+    const double s = sqrt(fma_rn(d2, d2, fma_rn(d1, d1, mul_rn(d0, d0))));
+    if (dep) {
+      if (tid == 0) window_cv_rec<double>(wd, 0, s, 0.0, s > 0 ? 0 : ABP_WFLAG_SINGULAR, true, st);
+      __syncthreads();
+      md_deposit<double, 1, 4>(g, fx, st, step0 + t, ra.log);
+    }
+    if (q == 0) {
+      // a4: the axis state (axis_eval with ul = 0) and the two corners
+      const double sa = here(s);
+      const double u = fma(sa, invD, u0);
+      int i0, i1;
+      double f;
+      bool clamped = false;
+      if (dep) {
+        i0 = st.i0[0];
+        i1 = st.i1[0];
+        f = st.f[0];
+        clamped = (st.cfl[0] >> 16) & 1;
+      } else if (per) {
+        const AxisSt<double> ax = axis_eval<double>(gd, wd.R[0], 0, here(sa), 0.0, false);
+        i0 = ax.i0;
+        i1 = ax.i1;
+        f = ax.f;
+      } else {
+        // out of range decided on the node index and the fraction's bits (an
+        // FP64 comparison costs as much as an addition)
+        const double fa = floor(u);
+        int k = (int)fa;
+        f = sub_rn(u, fa);
+        const bool below = k < 0 || !finite_bits(u) && !(u >= 0);
+        const bool above = !below && (k > n0 - 1 || (k == n0 - 1 && __double_as_longlong(f) != 0));
+        if (k > n0 - 2) {
+          k = n0 - 2;
+          f = add_rn(f, 1.0);
+        }
+        i0 = below ? 0 : above ? n0 - 2 : k;
+        f = below ? 0.0 : above ? 1.0 : f;
+        i1 = i0 + 1;
+        clamped = below || above;
+      }
+      double a0 = 0, a1 = 0;
+      if (lane < 2) {
+        const double wc = lane ? f : sub_rn(1.0, f);
+        const double2 r =
+            *reinterpret_cast<const double2 *>(rec + chk_node(gd, lane ? i1 : i0) * 16);
+        a0 = mul_rn(wc, r.x);
+        a1 = mul_rn(wc, r.y);
+      }
+      a0 = add_rn(a0, __shfl_xor_sync(0xffffffffu, a0, 1));
+      a1 = add_rn(a1, __shfl_xor_sync(0xffffffffu, a1, 1));
+      if (lane == 0) {
+        double dv = clamped ? 0.0 : a1;
+        if (wall) dv = add_rn(dv, wall_grad<double>(wd, 0, s));
+        dvs = dv;
+        V = a0;
+        s_last = s;
+        flags = (dep ? ABP_WFLAG_DEPOSIT : 0) | (clamped ? ABP_WFLAG_OOR : 0);
+      }
+    } else if (q == 1) {
+      const double sb = here(s);
+      const bool ok = sb > 0;
+      const double ir = rcp_fast<double>(sb);
+      if (lane == 0) {
+        us[0] = ok ? mul_rn(d0, ir) : 0.0;
+        us[1] = ok ? mul_rn(d1, ir) : 0.0;
+        us[2] = ok ? mul_rn(d2, ir) : 0.0;
+        sing = ok ? 0 : ABP_WFLAG_SINGULAR;
+      }
+    } else if (q == 2) {
+      const double sp = here(s);
+      if (lane == 0) dUs = mc.pot == ABP_POT_DOUBLE_WELL ? 4.0 * mc.dwa * sp * (sp * sp - mc.dwb2) : 0.0;
+    }
+    __syncwarp();
+    __syncthreads();
+    // a5 and the move of coordinate q
+    if (q < 3) {
+      const double dv = dvs, dt = add_rn(dv, dUs), u = us[q];
+      const bool keep_f = ra.forces || t == ra.nsteps - 1;
+      int bad = 0;
+      for (int i = lane; i < natoms; i += 32) {
+        const int ne = i == lane ? ne0 : wd.acnt[i];
+        const double w0 = i == lane ? w00 : ne > 0 ? terms[(size_t)i * kAtomTerms].w : 0.0;
+        const double w1 = i == lane ? w01 : ne > 1 ? terms[(size_t)i * kAtomTerms + 1].w : 0.0;
+        const double nzi = i == lane ? noise0 : nz[(size_t)t * nstride + i];
+        double f = 0;
+        if (ne > 0) f = fma_rn(mul_rn(w0, dt), u, f);
+        if (ne > 1) f = fma_rn(mul_rn(here(w1), dt), u, f);
+        double xi = x[i];
+        if (tout) {
+          double *o = reinterpret_cast<double *>(tout + (long long)t * a.tstride + i);
+          o[q] = xi;
+          if (q == 0) o[3] = xs[3 * natoms + i];
+        }
+        if (keep_f) {
+          const double db = here(dv);
+          double b = 0;
+          if (ne > 0) b = fma_rn(mul_rn(w0, db), u, b);
+          if (ne > 1) b = fma_rn(mul_rn(here(w1), db), u, b);
+          double *o = reinterpret_cast<double *>(fout + (ra.forces ? (long long)t * ra.fstride : 0) + i);
+          if (fmode == ABP_FORCES_ACCUMULATE) {
+            o[q] += b;
+          } else {
+            o[q] = b;
+            if (q == 0) o[3] = 0.0;
+          }
+        }
+        xi = add_rn(xi, fma_rn(mc.c1, f, nzi));
+        x[i] = xi;
+        bad |= finite_bits(xi) ? 0 : 1;
+      }
+      bad = __any_sync(0xffffffffu, bad);
+      if (lane == 0) bads[q] = bad;
+      __syncwarp();
+    }
+    last = t;
+  }
+  __syncthreads();
+  for (int i = tid; i < natoms; i += kLineThreads)
+    cio[i] = make_rec<double>(xs[i], xs[natoms + i], xs[2 * natoms + i], xs[3 * natoms + i]);
+  if (tid == 0 && last >= 0) {
+    WalkerState ws;
+    for (int k = 0; k < 3; ++k) ws.s[k] = ws.dV[k] = 0.0;
+    ws.s[0] = s_last;
+    ws.dV[0] = dvs;
+    ws.V = V;
+    ws.flags = stopped ? ABP_WFLAG_NONFINITE : flags | sing;
+    ws.pad = 0;
+    ws.step = step0 + last;
+    *wd.state = ws;
+  }
+}
+
 }  // namespace
 
 int md_group_bytes(const WalkerDev &hd, int fp64) {
   const int fixed = fp64 ? md_fixed_bytes<double>() : md_fixed_bytes<float>();
   return align32(fixed + md_layout(hd.natoms, hd.cv, hd.g.d, fp64).total);
+}
+
+size_t md_noise_bytes(int nw, int max_atoms, int nsteps) { return (size_t)nw * nsteps * 3 * max_atoms * 8; }
+
+cudaError_t launch_md_line(const MdRunArgs &a, int max_atoms, void *noise, LaunchTimer *tm, cudaStream_t st) {
+  const RunArgs &r = a.r;
+  const int stride = 3 * max_atoms;
+  const long long items = (long long)r.nsteps * max_atoms;
+  if (tm) tm->begin("k_md_noise", st);
+  k_md_noise<<<dim3((unsigned)((items + 127) / 128), r.nw), 128, 0, st>>>(r.table, a.md, r.step0, r.nsteps, stride,
+                                                                          static_cast<double *>(noise));
+  if (tm) tm->end("k_md_noise", st);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const size_t smem = line_layout(max_atoms).total;
+  e = smem_attr(reinterpret_cast<const void *>(k_md_line), smem);
+  if (e != cudaSuccess) return e;
+  NvtxRange nv("k_md_line");
+  if (tm) tm->begin("k_md_line", st);
+  k_md_line<<<r.nw, kLineThreads, smem, st>>>(a, static_cast<const double *>(noise), stride);
+  if (tm) tm->end("k_md_line", st);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_md(const MdRunArgs &a, int fp64, int dim, bool fast, cudaStream_t st) {
