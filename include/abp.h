@@ -248,8 +248,8 @@ abp_status abp_forces(abp_ctx *ctx, abp_walker *const *walkers, int n, void *for
  * walkers with their own grids, equal per step and walker to abp_step followed
  * by abp_forces. One launch for short calls; longer ones run in three launches
  * over scratch of at most 240 MB from a pool that the library keeps per device
- * while it has contexts there (without that memory, one launch: the same
- * results). Coordinates of step t at record
+ * while it has contexts there (without that memory, or while the stream is
+ * being captured, one launch: the same results). Coordinates of step t at record
  * coord_offsets_dev[w] + t * coord_step_stride + i; forces written (by mode)
  * at force_offsets_dev[w] + t * force_step_stride + i. Walkers that share a
  * grid are rejected (use abp_step). */

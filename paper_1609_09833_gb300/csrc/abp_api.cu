@@ -201,9 +201,10 @@ constexpr int kLineMaxAtoms = 2048;          // atoms of a walker of k_md_line (
 constexpr size_t kReadoutChunk = 32u << 20;  // staging bytes of a readout
 
 // The library's memory pool of a device, shared by its contexts there: made
-// by the first call that needs scratch, given back with the last context. It
-// keeps up to kPoolKeep bytes between calls (mapping them again on every call
-// took ~0.3 ms).
+// with the first of them (so that no later call makes one while a stream is
+// being captured), given back with the last. It holds no memory until a call
+// takes scratch and keeps up to kPoolKeep bytes between calls (mapping them
+// again on every call took ~0.3 ms).
 constexpr int kMaxDevices = 64;
 struct DevicePool {
   cudaMemPool_t pool = nullptr;
@@ -221,43 +222,45 @@ void pool_context(int device, int delta) {
     cudaMemPoolDestroy(p.pool);
     p.pool = nullptr;
   }
+  if (delta <= 0 || p.pool) return;
+  cudaMemPoolProps pr{};
+  pr.allocType = cudaMemAllocationTypePinned;
+  pr.location.type = cudaMemLocationTypeDevice;
+  pr.location.id = device;
+  uint64_t keep = kPoolKeep;
+  if (cudaMemPoolCreate(&p.pool, &pr) != cudaSuccess) {
+    p.pool = nullptr;
+  } else if (cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaMemPoolDestroy(p.pool);
+    p.pool = nullptr;
+  }
+  if (!p.pool) cudaGetLastError();  // calls then take the forms without scratch
 }
 
 cudaError_t pool_get(int device, cudaMemPool_t *out) {
   *out = nullptr;
   if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(g_pool_mu);
-  DevicePool &p = g_pools[device];
-  cudaError_t e = cudaSuccess;
-  if (!p.pool) {
-    cudaMemPoolProps pr{};
-    pr.allocType = cudaMemAllocationTypePinned;
-    pr.location.type = cudaMemLocationTypeDevice;
-    pr.location.id = device;
-    uint64_t keep = kPoolKeep;
-    e = cudaMemPoolCreate(&p.pool, &pr);
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e != cudaSuccess && p.pool) {
-      cudaMemPoolDestroy(p.pool);
-      p.pool = nullptr;
-    }
-  }
-  *out = p.pool;
-  return e;
+  *out = g_pools[device].pool;
+  return *out ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 
 // Scratch of one call, ordered on the context's stream: taken from the
 // device's pool and returned to it when the object goes out of scope, behind
 // the work queued so far. Calls on different streams or threads never share a
-// block, and under stream capture the block belongs to the graph. p is null
-// if there is no memory (err says why).
+// block. p is null if there is no memory (err says why), and always while the
+// stream is being captured: the block would be a memory node, and a graph
+// with one can be neither cloned nor nested nor instantiated twice.
 struct Scratch {
   void *p = nullptr;
   cudaError_t err = cudaSuccess;
   cudaStream_t st;
   Scratch(abp_ctx *ctx, size_t bytes) : st(ctx->stream) {
     cudaMemPool_t pool = nullptr;
-    err = pool_get(ctx->device, &pool);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    err = cudaStreamIsCapturing(st, &cs);
+    if (err == cudaSuccess && cs != cudaStreamCaptureStatusNone) err = cudaErrorStreamCaptureUnsupported;
+    if (err == cudaSuccess) err = pool_get(ctx->device, &pool);
     if (err == cudaSuccess) err = cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), pool, st);
     if (err != cudaSuccess) {
       cudaGetLastError();

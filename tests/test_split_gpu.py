@@ -150,3 +150,64 @@ def test_many_walkers_give_the_bits_of_one(nw):
         na = specs[i]["natoms"]
         f, g, _ = _run(abp, [specs[i]], frames[:, offs[i]:offs[i] + na], abp.ABP_FORCES_OVERWRITE, [9])
         assert np.array_equal(f, F[:, offs[i]:offs[i] + na]) and np.array_equal(g[0], G[i])
+
+
+@pytest.mark.parametrize("form", ["sweep", "pocket", "double_well"])
+def test_captured_calls_take_forms_without_scratch(form):
+    """A long abp_run and an FP64 abp_md_run captured in a CUDA graph give the
+    bits of the direct calls, and the graph can be cloned (one with memory
+    nodes cannot)."""
+    import ctypes
+
+    from paper_1609_09833_gb300 import abp
+
+    T, runs = 70, []
+    md = form == "double_well"
+    well = {"natoms": 16, "cvs": [{"type": "com_dist", "a": np.arange(8), "b": np.arange(8, 16)}],
+            "grid": synth.grid((-2.0,), (4.0,), (512,), (False,)), "hill": synth.hill(0.8, (0.05,), 10, 8.0)}
+    specs = [well] if md else _specs(form)
+    x0 = np.random.default_rng(4).uniform(0.0, 1.5, size=(1, specs[0]["natoms"], 3))
+    frames = x0 if md else _frames(specs, 2 * T, 7)
+    for captured in (False, True):
+        ctx = abp.Context(0)
+        try:
+            ws = ctx.make_walkers(specs, precision=abp.ABP_PREC_FP64 if md else abp.ABP_PREC_FP32_COMP)
+            x = (torch.as_tensor(np.concatenate([frames, np.ones_like(frames[..., :1])], 2)) if md
+                 else abp.to_records(frames)).cuda()
+            A = x.shape[1]
+            F = torch.zeros_like(x)
+            offs = torch.tensor(synth.offsets_of(specs), dtype=torch.int64, device="cuda")
+
+            def call(t):
+                if md:
+                    abp.abp_md_run(ctx.handle, ws, x[0], abp.ABP_F64, offs, synth.md_double_well(seed=3),
+                                   np.zeros(1, dtype=np.uint32), step0=t, nsteps=T)
+                else:
+                    abp.abp_run(ctx.handle, ws, x[t:], abp.ABP_F32, offs, A, F[t:], offs, A,
+                                abp.ABP_FORCES_OVERWRITE, t, T)
+
+            call(0)  # (caches the walker table)
+            if captured:
+                s = torch.cuda.Stream()
+                torch.cuda.synchronize()
+                ctx.set_stream(s.cuda_stream)
+                g = torch.cuda.CUDAGraph(keep_graph=True)
+                with torch.cuda.graph(g, stream=s):
+                    call(T)
+                rt, copy = ctypes.CDLL("libcudart.so.13"), ctypes.c_void_p()
+                assert rt.cudaGraphClone(ctypes.byref(copy), ctypes.c_void_p(g.raw_cuda_graph())) == 0
+                assert rt.cudaGraphDestroy(copy) == 0
+                g.instantiate()
+                g.replay()
+                torch.cuda.synchronize()
+                ctx.set_stream(torch.cuda.current_stream().cuda_stream)
+            else:
+                call(T)
+            torch.cuda.synchronize()
+            runs.append((x.cpu().numpy(), F.cpu().numpy(), [ctx.bias(w) for w in ws]))
+        finally:
+            torch.cuda.synchronize()
+            ctx.close()
+    assert np.array_equal(runs[0][0], runs[1][0]) and np.array_equal(runs[0][1], runs[1][1])
+    for a, b in zip(runs[0][2], runs[1][2]):
+        assert np.array_equal(a, b)
