@@ -467,7 +467,7 @@ def bench_paper_rmsd(abp, synth, torch, dev):
                 "stencil_nodes": box,
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                              "frac": achieved / peaks["hbm_gbs"], "bytes_per_walker_step": per_step,
-                             "kernel": "k_win<float> (windowed form)", "peak_source": src},
+                             "kernel": "k_sp_cv, k_sp_hist, k_sp_force (split form)", "peak_source": src},
                 "cpu_baseline": cpu}
     finally:
         torch.cuda.synchronize()
@@ -500,7 +500,7 @@ def bench_uneven(abp, synth, torch, dev, sm_mhz, fp32):
         flops = nw * C * 40 * 400 * CN_PAIR_FLOPS
         achieved = flops / (ms / 1e3) / 1e12
         peak = fp32.at(sm_mhz)
-        # the same launch replayed from a CUDA graph
+        # the same call replayed from a CUDA graph (captured calls run in k_run)
         s = torch.cuda.Stream()
         ctx.set_stream(s.cuda_stream)
         g = torch.cuda.CUDAGraph()
@@ -534,7 +534,7 @@ def bench_uneven(abp, synth, torch, dev, sm_mhz, fp32):
 
         cpu = oracle_rate(ostep, ns, 3.0, f"one MD step of the first {ns} walkers")
         return {"workload": "1000 walkers (40% 1D 1024, 50% 2D 128^2/256^2/512^2, 10% 3D 64^3), CN 40x400, "
-                            "jitter frames, one launch per 25 MD steps",
+                            "jitter frames, one call per 25 MD steps",
                 "value": nw * C / (ms / 1e3), "unit": "bias steps/s", "ms_per_launch": ms,
                 "graph_replay": {"value": nw * C / (ms_graph / 1e3), "ms_per_launch": ms_graph},
                 "plain": {"value": plain, "ratio": nw * C / (ms / 1e3) / plain,
@@ -542,8 +542,9 @@ def bench_uneven(abp, synth, torch, dev, sm_mhz, fp32):
                 "cpu_baseline": cpu,
                 "tuned": tuned["best"],
                 "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                             "frac": achieved / peak, "kernel": "k_run / k_run_lean (per-step form, CN pairs)",
-                             "traffic": captured_traffic("k_run_uneven1000", nw * C),
+                             "frac": achieved / peak,
+                             "kernel": "k_sp_cn, k_sp_chain, k_sp_cnf (split form); the pairs are k_sp_cn's",
+                             "traffic": captured_traffic("split_uneven1000", nw * C),
                              "flops_per_pair": CN_PAIR_FLOPS, "peak_source": fp32.source(sm_mhz)}}
     finally:
         torch.cuda.synchronize()
@@ -553,8 +554,8 @@ def bench_uneven(abp, synth, torch, dev, sm_mhz, fp32):
 def bench_shared(abp, synth, torch, dev, sm_mhz, fp32):
     """32 walkers on one shared 256^3 grid, 200 x 10,000-atom CN each: the
     closed loop (free overdamped Langevin of every atom under the bias, the
-    phased form's five launches plus the move per MD step), replayed as a
-    CUDA graph of C steps; the open-loop replay of jitter frames beside it;
+    phased form's three launches per MD step, six on a step that deposits),
+    replayed as a CUDA graph of C steps; the open-loop replay of jitter frames beside it;
     the pair kernel's own time from the library's per-kernel timing."""
     ctx = abp.Context(dev)
     try:
@@ -635,8 +636,8 @@ def bench_shared(abp, synth, torch, dev, sm_mhz, fp32):
                             "atoms, 6 nm periodic box, stride 10; closed loop (free overdamped Langevin, mu = 0.05), "
                             "10 MD steps per call, CUDA-graph replay",
                 "value": nw * C / (ms_graph / 1e3), "unit": "bias steps/s", "ms_per_md_step": ms_graph / C,
-                "value_direct_calls": nw * C / (ms_direct / 1e3), "gpu_launches_per_md_step": 6,
-                "open_loop_replay": {"value": nw * C / (ms_open / 1e3), "gpu_launches_per_md_step": 5},
+                "value_direct_calls": nw * C / (ms_direct / 1e3), "gpu_launches_per_md_step": 3 + 3 * (1 / 10),
+                "open_loop_replay": {"value": nw * C / (ms_open / 1e3), "gpu_launches_per_md_step": 3 + 3 * (1 / 10)},
                 "kernel_ms_per_md_step": {k: v[1] / max(v[0], 1) for k, v in times.items()},
                 "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                              "frac": achieved / peak, "kernel": "k_big_cn (pair kernel), its own CUDA-event time",
@@ -822,8 +823,8 @@ def bench_serve(abp, synth, torch, dev, seconds=2.0, rate=20_000.0):
 KERNEL_SOURCES = {
     "k_md_mb64": ["abp_md.cu", "abp_md.cuh", "abp_window_ops.cuh", "abp_device.cuh", "abp_internal.cuh",
                   "abp_launch.h"],
-    "k_win_mb64": ["abp_kernels.cu", "abp_window_ops.cuh", "abp_device.cuh", "abp_internal.cuh", "abp_launch.h"],
-    "k_run_uneven1000": ["abp_kernels.cu", "abp_window_ops.cuh", "abp_device.cuh", "abp_internal.cuh",
+    "split_mb64": ["abp_split.cu", "abp_window_ops.cuh", "abp_device.cuh", "abp_internal.cuh", "abp_launch.h"],
+    "split_uneven1000": ["abp_split.cu", "abp_window_ops.cuh", "abp_device.cuh", "abp_internal.cuh",
                          "abp_launch.h"],
     "k_big_cn_shared256": ["abp_big.cu", "abp_md.cuh", "abp_device.cuh", "abp_internal.cuh", "abp_launch.h"],
 }
@@ -1051,12 +1052,12 @@ def main():
                 "us_per_walker_step": 1e3 * kernel_ms / C}
     open_achieved = BYTES_PER_WALKER_STEP * NW * C / (open_ms / 1e3) / 1e9
     open_loop = {"workload": "the same 64 walkers replaying 4000 recorded open-loop frames (147 MB, larger than "
-                             "L2, cycled), windowed form", "value": NW * C / (open_ms / 1e3), "unit": UNIT,
+                             "L2, cycled), split form", "value": NW * C / (open_ms / 1e3), "unit": UNIT,
                  "ms_per_launch": open_ms, "md_steps_per_launch": C, "launch_shape": tuned,
                  "roofline": {"bound": "hbm", "achieved": open_achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                               "frac": open_achieved / peaks["hbm_gbs"],
-                              "traffic": captured_traffic("k_win_mb64", NW * C),
-                              "kernel": "k_win<float> (windowed form)", "peak_source": psrc,
+                              "traffic": captured_traffic("split_mb64", NW * C),
+                              "kernel": "k_sp_cv, k_sp_chain, k_sp_force (split form)", "peak_source": psrc,
                               "bytes_per_walker_step": BYTES_PER_WALKER_STEP}}
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:

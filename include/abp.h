@@ -303,8 +303,11 @@ typedef struct {
 } abp_md_desc;
 
 /* nsteps closed-loop MD steps step0..step0+nsteps-1 of n walkers in one
- * launch. coords_dev holds each walker's atoms at step0 (records at
- * coord_offsets_dev[w] + i, dtype as for abp_run) and receives them after
+ * launch (FP64 walkers of one COM distance, at most one a multiprocessor: a
+ * pair of launches per block of steps whose noise fits 64 MB of the pool's
+ * scratch; without it, one launch: the same results). coords_dev holds each
+ * walker's atoms at step0 (records at coord_offsets_dev[w] + i, dtype as for
+ * abp_run) and receives them after
  * the last step's move (in place). streams (host, n values) are the walkers'
  * noise streams. Optional outputs (NULL to skip): traj_dev, the coordinates
  * each step's bias was evaluated at (records at traj_offsets_dev[w] +
@@ -313,7 +316,7 @@ typedef struct {
  * abp_forces delivers the last step's). Walkers whose CVs are COM
  * distances, dihedrals or RMSDs run one warp each (steps chained on the
  * device); walkers of the phased form (a shared grid or a large walker) run
- * their step's launches followed by the move, and take ABP_POT_NONE only.
+ * their step's launches, the last of which moves the atoms, and take ABP_POT_NONE only.
  * Other walkers (a coordination number in the fused form) are rejected with
  * ABP_ERR_UNSUPPORTED. A walker that meets non-finite coordinates stops
  * there (its state reports ABP_WFLAG_NONFINITE; abp_sync returns
