@@ -467,7 +467,9 @@ def bench_paper_rmsd(abp, synth, torch, dev):
                 "stencil_nodes": box,
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                              "frac": achieved / peaks["hbm_gbs"], "bytes_per_walker_step": per_step,
-                             "kernel": "k_sp_cv, k_sp_hist, k_sp_force (split form)", "peak_source": src},
+                             "kernel": "k_sp_cv, k_sp_hist, k_sp_force (split form)", "peak_source": src,
+                             "note": "a hill's nodes stay in registers over up to 64 hills, so the counted bytes "
+                                     "of a hill do not all reach HBM"},
                 "cpu_baseline": cpu}
     finally:
         torch.cuda.synchronize()
