@@ -251,7 +251,9 @@ abp_status abp_forces(abp_ctx *ctx, abp_walker *const *walkers, int n, void *for
  * while it has contexts there (without that memory, or while the stream is
  * being captured, one launch: the same results). Coordinates of step t at record
  * coord_offsets_dev[w] + t * coord_step_stride + i; forces written (by mode)
- * at force_offsets_dev[w] + t * force_step_stride + i. Walkers that share a
+ * at force_offsets_dev[w] + t * force_step_stride + i, in step order where
+ * the steps' records are the same (a stride of 0) or overlap (a stride shorter
+ * than a walker: a launch per step). Walkers that share a
  * grid are rejected (use abp_step). */
 abp_status abp_run(abp_ctx *ctx, abp_walker *const *walkers, int n, const void *coords_dev, int coords_dtype,
                    const int64_t *coord_offsets_dev, int64_t coord_step_stride, void *forces_dev,

@@ -8,7 +8,6 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -1152,7 +1151,7 @@ constexpr size_t kSplitScratch = 240u << 20;  // (below kPoolKeep, so that the p
 static abp_status run_split(abp_ctx *ctx, const std::vector<abp_walker *> &ws, const TableEntry *table, bool win,
                             SplitArgs a, int nsteps, bool *done) {
   SplitShape shape;
-  int jrec = 0, max_atoms = 0;
+  int jrec = 0;
   size_t words = 0;
   for (const abp_walker *w : ws) {
     split_shape(w->hd, win, &shape);
@@ -1160,9 +1159,8 @@ static abp_status run_split(abp_ctx *ctx, const std::vector<abp_walker *> &ws, c
       jrec = std::max(jrec, split_jac_records(w->hd));
       words = std::max(words, (size_t)split_term_words(w->hd));
     }
-    max_atoms = std::max(max_atoms, w->hd.natoms);
   }
-  a.serial = a.forces && std::llabs(a.fstride) < max_atoms;
+  a.serial = a.forces && a.fstride == 0;
   a.jstride = jrec;
   a.term_stride = words;
   // per walker and step its record and gradient records, per walker its atoms' terms
@@ -1233,6 +1231,23 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     return fail(ABP_ERR_INVALID_ARG, "FP64 coordinate and force buffers must be 32-byte aligned");
   st = set_device(ctx);
   if (st) return st;
+  // Force records of a walker's steps that overlap without coinciding: inside
+  // a launch other threads may be storing another step's atom in the same
+  // record, so every step gets launches of its own, which the stream orders
+  // (a stride of 0 needs none of this: one thread keeps an atom's record).
+  if (forces && nsteps > 1 && fstride != 0) {
+    int64_t max_atoms = 0;
+    for (int i = 0; i < n; ++i) max_atoms = std::max<int64_t>(max_atoms, walkers[i]->hd.natoms);
+    if (fstride > -max_atoms && fstride < max_atoms) {
+      const int64_t rsz = fp64 ? 32 : 16;
+      for (int t = 0; t < nsteps; ++t)
+        if ((st = run_common(ctx, walkers, n, static_cast<const unsigned char *>(coords) + t * cstride * rsz, cdt, coff,
+                             cstride, static_cast<unsigned char *>(forces) + t * fstride * rsz, foff, fstride, mode,
+                             step0 + t, 1)))
+          return st;
+      return ABP_OK;
+    }
+  }
   // three forms: windowed (k_win, one launch per grid dimension), per-step
   // fused (k_run), phased (big)
   std::vector<abp_walker *> ww[3], fw, bw;

@@ -92,7 +92,7 @@ struct SplitArgs {
   const long long *foff;
   long long fstride;
   int mode;
-  int serial;          // the force records of a walker's steps overlap: added in step order
+  int serial;          // every step writes the same force records (stride 0): in step order, an atom a thread
   int last;            // the call's last block
   int chunk;           // steps per warp of k_sp_cn (set by the launcher)
   long long step0;     // MD step of the call's first step

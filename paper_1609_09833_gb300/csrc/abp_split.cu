@@ -886,8 +886,8 @@ __device__ __forceinline__ float4 *force_out(const SplitArgs &a, const WalkerDev
 // A window's forces from its step records: the Jacobian factors scaled by
 // dV/ds into shared memory (as finish_lookup scales them), then one atom per
 // thread over every nl-th step, its terms (the walker's table) in registers.
-// a.serial: the steps' records overlap, so one CTA per walker adds them in
-// step order.
+// a.serial: every step writes the same records, so one CTA per walker takes
+// the windows in turn, an atom always on the same thread.
 struct ForceRec {
   float jac[kMaxCv * 12];
 };
