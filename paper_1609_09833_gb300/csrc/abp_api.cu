@@ -1867,18 +1867,35 @@ static abp_status readout_by_host(abp_ctx *ctx, const abp_grid *g, void *dst, in
   return ABP_OK;
 }
 
+// st waits for the work queued so far on the default stream (and, by that
+// stream's own rule, on every blocking stream), as a cudaMemcpy does: a side
+// stream may be one that would not.
+static cudaError_t wait_default_stream(cudaStream_t st) {
+  if (!st || st == cudaStreamLegacy) return cudaSuccess;
+  cudaEvent_t ev;
+  cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) return e;
+  e = cudaEventRecord(ev, cudaStreamLegacy);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev, 0);
+  cudaEventDestroy(ev);
+  return e;
+}
+
 abp_status abp_bias_readout(abp_ctx *ctx, const abp_grid *g, void *dst, int dst_is_device, int dtype) {
   if (!ctx || !g || !dst || g->ctx != ctx) return fail(ABP_ERR_INVALID_ARG, "bad argument");
   if (dtype != ABP_F32 && dtype != ABP_F64) return fail(ABP_ERR_INVALID_ARG, "bad dtype");
   abp_status st = set_device(ctx);
   if (st) return st;
   // converted on the device into a staging block, copied from there (the copy
-  // checks the destination as it always did: its kind, size and alignment)
+  // checks the destination as it always did: its kind, size and alignment);
+  // into device memory behind what the caller has queued there, a fill of dst
+  // on the default stream for instance
   const GridDev &gd = g->g;
   const size_t node = (size_t)(1 + gd.d) * (dtype == ABP_F64 ? 8 : 4);
   const long long chunk = std::min(gd.nodes, (long long)(kReadoutChunk / node));
   Scratch stage(ctx, (size_t)chunk * node);
   if (!stage.p) return readout_by_host(ctx, g, dst, dst_is_device, dtype);
+  if (dst_is_device) CUDA_TRY(wait_default_stream(ctx->stream));
   for (long long i = 0; i < gd.nodes; i += chunk) {
     const long long c = std::min(chunk, gd.nodes - i);
     CUDA_TRY(launch_readout(gd, i, c, stage.p, dtype == ABP_F64, ctx->stream));
