@@ -990,8 +990,8 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
       }
     }
   }
-  if (st == ABP_OK && w->big && big_cn_smem(hd) > 200 * 1024)
-    st = fail(ABP_ERR_UNSUPPORTED, "a coordination number with more than ~2000 A atoms is not built");
+  if (st == ABP_OK && w->big && big_cn_too_large(hd))
+    st = fail(ABP_ERR_UNSUPPORTED, "a coordination number with more than 1828 A atoms is not built");
   if (st == ABP_OK && w->big && big_part_bytes(hd) > 0) {
     // (not counted against the budget, which is for grids and walkers)
     if (cudaMalloc(&p, big_part_bytes(hd)) != cudaSuccess) {

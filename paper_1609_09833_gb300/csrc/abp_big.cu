@@ -960,6 +960,15 @@ cudaError_t read_hill_heads(const WalkerDev *const *wd_host, int n, double *s3h,
   return e;
 }
 
+// The phased form takes coordination numbers of up to kBigMaxA A atoms (200 KB
+// at 16 + 8 x 12 bytes an atom, the shared memory of a pair CTA of eight
+// warps; the CTAs of two warps stay below that).
+constexpr int kBigMaxA = 200 * 1024 / (16 + 8 * 12);
+bool big_cn_too_large(const WalkerDev &hd) {
+  const int k = big_cn_index(hd);
+  return k >= 0 && hd.cv[k].na > kBigMaxA;
+}
+
 size_t big_cn_smem(const WalkerDev &hd) {
   int k = big_cn_index(hd);
   if (k < 0) return 0;

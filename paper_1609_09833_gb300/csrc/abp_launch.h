@@ -208,6 +208,7 @@ size_t big_nterm_offset(const WalkerDev &hd);
 int big_cn_count(const WalkerDev &hd);
 int big_chunks(const WalkerDev &hd);
 size_t big_cn_smem(const WalkerDev &hd);
+bool big_cn_too_large(const WalkerDev &hd);
 cudaError_t launch_big_step(const BigArgs &a, cudaStream_t st);
 // Hill records handed to a grid: one per record, in waves of disjoint boxes.
 struct HillDev {
