@@ -184,6 +184,7 @@ struct abp_walker {
   bool big = false;    // runs in the phased form (shared grid, or too large for a walker group)
   bool win = false;    // runs in the windowed form of the fused kernel (COM distance / dihedral CVs)
   bool has_rmsd = false;
+  bool group_fits = false;  // a walker group of the default width fits one SM's shared memory
   // the closed-loop kernel's register-fed form applies: FP32 WT walkers of at
   // most 64 atoms of at most two a5 terms each, COM groups of at most 16
   // atoms, the other CVs dihedrals
@@ -403,12 +404,15 @@ abp_status step_shape(const abp_ctx *ctx, bool cn, int g, int gb, int tb, int *G
   return ABP_OK;
 }
 
+// Default threads of a walker group: windowed form, coordination numbers, others.
+constexpr int kWinGroup = 256, kCnGroup = 128, kRunGroup = 32;
+
 abp_status pick_shape(const abp_ctx *ctx, abp_walker *const *walkers, int n, int fp64, int nsteps, bool window,
                       int *G, int *gpc, int *group_bytes, int *tile_budget) {
   bool cn = false;
   for (int i = 0; i < n; ++i) cn = cn || walkers[i]->has_cn;
   if (window) {
-    const int g = ctx->tune_G ? ctx->tune_G : 256;
+    const int g = ctx->tune_G ? ctx->tune_G : kWinGroup;
     int gb = 0;
     for (int i = 0; i < n; ++i) gb = std::max(gb, run_group_bytes(walkers[i]->hd, fp64, g, 0, true));
     const int smem_max = 227 * 1024;
@@ -421,7 +425,7 @@ abp_status pick_shape(const abp_ctx *ctx, abp_walker *const *walkers, int n, int
     *tile_budget = 0;
     return ABP_OK;
   }
-  const int g = ctx->tune_G ? ctx->tune_G : (cn ? 128 : 32);
+  const int g = ctx->tune_G ? ctx->tune_G : (cn ? kCnGroup : kRunGroup);
   int fixed = group_fixed_bytes(fp64);
   int tb = 0;
   // Measured on the 64-walker workload, one warp per walker: reloading and
@@ -931,6 +935,8 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
   // for one shared-memory walker group (FP32, at most one CN)
   w->big = grid->desc.shared || run_group_bytes(hd, fp64, 32, 0, false) > 227 * 1024;
   w->win = !w->big && window_eligible(hd, fp64);
+  w->group_fits = run_group_bytes(hd, fp64, w->win ? kWinGroup : w->has_cn ? kCnGroup : kRunGroup, 0, w->win) <=
+                  227 * 1024;
   if (w->win) {
     // the closed-loop form's a5 term tables (read, not rebuilt, by each launch)
     std::vector<int> tcnt;
@@ -1276,7 +1282,8 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1;
     bool mabp = false;
     for (size_t i = 0; split && i < lw.size(); ++i) {
-      split = split_eligible(lw[i]->hd, win);
+      // (a walker whose group does not fit is refused below, whatever the form)
+      split = lw[i]->group_fits && split_eligible(lw[i]->hd, win);
       mabp = mabp || lw[i]->hd.method == ABP_METHOD_MABP;
     }
     if (split) {
