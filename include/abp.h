@@ -165,7 +165,10 @@ typedef struct {
 /* Creates a context on `device`, issuing work on `cuda_stream` (a
  * cudaStream_t; NULL = the legacy default stream). hbm_budget_bytes caps the
  * bytes the context may allocate for grids and walkers (0 = no cap): an
- * allocation beyond it fails with ABP_ERR_ADMISSION. */
+ * allocation beyond it fails with ABP_ERR_ADMISSION. Outside it are the scratch
+ * of a call (at most 240 MB, of which the device's contexts together keep up
+ * to 256 MB between calls and give it back with the last of them) and small
+ * tables. */
 abp_status abp_ctx_create(abp_ctx **out, int device, void *cuda_stream, size_t hbm_budget_bytes);
 abp_status abp_ctx_set_stream(abp_ctx *ctx, void *cuda_stream);
 /* Bytes currently allocated against the budget. */

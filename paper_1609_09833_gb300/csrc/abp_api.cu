@@ -689,8 +689,6 @@ abp_status upload(abp_walker *w, const void *src, size_t bytes, void **dst) {
 void walker_free(abp_walker *w) {
   for (auto &a : w->allocs) dev_free(w->ctx, a.first, a.second);
   w->allocs.clear();
-  if (w->hd.bpart) cudaFree(w->hd.bpart);
-  w->hd.bpart = nullptr;
 }
 
 abp_status check_indices(const int32_t *idx, int n, int natoms, const char *what, int k) {
@@ -998,15 +996,9 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
   }
   if (st == ABP_OK && w->big && big_cn_too_large(hd))
     st = fail(ABP_ERR_UNSUPPORTED, "a coordination number with more than 1828 A atoms is not built");
-  if (st == ABP_OK && w->big && big_part_bytes(hd) > 0) {
-    // (not counted against the budget, which is for grids and walkers)
-    if (cudaMalloc(&p, big_part_bytes(hd)) != cudaSuccess) {
-      cudaGetLastError();
-      st = fail(ABP_ERR_OOM, "cudaMalloc of %zu bytes for partial sums", big_part_bytes(hd));
-    } else {
-      hd.bpart = p;
-    }
-  }
+  if (st == ABP_OK && w->big && big_part_bytes(hd) > 0 &&
+      (st = walker_alloc(w, big_part_bytes(hd), &p)) == ABP_OK)
+    hd.bpart = p;
   if (st == ABP_OK && w->big) {
     // the force phase's per-atom term table, into the walker's scratch
     std::vector<int32_t> terms;
