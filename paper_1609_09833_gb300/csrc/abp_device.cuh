@@ -1801,13 +1801,18 @@ __device__ __forceinline__ void mabp_bias(const WalkerDev &wd, const Real *acc, 
   for (int k = 0; k < wd.g.d; ++k) dv[k] = (Real)wd.mabp_g * acc[1 + k] / den;
 }
 
-// dU/ds_k of the CV range limit: kwall (s - smax_k) above smax_k, else 0.
+// dU/ds_k of the CV range limit: kwall (s + sl - smax_k) above smax_k, else 0.
+// (An FP32 CV's high part alone is a few units in the last place off: 2.2e-7
+// nm of a 3.6 nm COM distance, 8e-8 with sl.)
 template <typename Real>
-__device__ __forceinline__ Real wall_grad(const WalkerDev &wd, int k, Real s) {
-  if constexpr (sizeof(Real) == 4)
-    return (wd.kwall_f > 0.f && s > wd.smax_f[k]) ? mul_rn(wd.kwall_f, sub_rn(s, wd.smax_f[k])) : 0.f;
-  else
+__device__ __forceinline__ Real wall_grad(const WalkerDev &wd, int k, Real s, Real sl = (Real)0) {
+  if constexpr (sizeof(Real) == 4) {
+    if (!(wd.kwall_f > 0.f)) return 0.f;
+    const float e = add_rn(sub_rn(s, wd.smax_f[k]), sl);
+    return e > 0.f ? mul_rn(wd.kwall_f, e) : 0.f;
+  } else {
     return (wd.kwall > 0 && s > (Real)wd.smax[k]) ? mul_rn((Real)wd.kwall, sub_rn(s, (Real)wd.smax[k])) : (Real)0;
+  }
 }
 
 // a4: V and dV/ds_k at s after the deposit, by the group's first warp: lane c
@@ -1843,9 +1848,8 @@ __device__ void interp_step(const Grp &g, GroupFixed<Real> *fx, const GroupLayou
       }
       fx->V = acc[0];
       for (int k = 0; k < d; ++k) {
-        // the wall acts on the CV's high part, as in finish_lookup
-        const Real dv =
-            add_rn(((fx->clamped >> k) & 1) ? (Real)0 : acc[1 + k], wall_grad<Real>(fx->wd, k, fx->sh[k]));
+        const Real dv = add_rn(((fx->clamped >> k) & 1) ? (Real)0 : acc[1 + k],
+                               wall_grad<Real>(fx->wd, k, fx->sh[k], fx->sl[k]));
         fx->dvds[k] = dv;
         fx->dV[k] = dv;
       }

@@ -470,7 +470,7 @@ __device__ __forceinline__ void step_lookup(const WalkerDev &wd, Step *sp) {
   sp->V = acc[0];
 #pragma unroll
   for (int k = 0; k < DIM; ++k)
-    sp->dv[k] = add_rn(((clamped >> k) & 1) ? 0.f : acc[1 + k], wall_grad<float>(wd, k, s.s[k]));
+    sp->dv[k] = add_rn(((clamped >> k) & 1) ? 0.f : acc[1 + k], wall_grad<float>(wd, k, s.s[k], sp->sl[k]));
 }
 
 // The walker's state after the call's last step.
@@ -841,7 +841,7 @@ __device__ __forceinline__ void hist_body(const Grp &g, GroupFixed<float> *fx, H
       s.V = V;
 #pragma unroll
       for (int k = 0; k < DIM; ++k)
-        s.dv[k] = add_rn(((s.clamped >> k) & 1) ? 0.f : dv[k], wall_grad<float>(wd, k, s.s[k]));
+        s.dv[k] = add_rn(((s.clamped >> k) & 1) ? 0.f : dv[k], wall_grad<float>(wd, k, s.s[k], s.sl[k]));
     }
     t0 += nt;
   }
