@@ -693,8 +693,9 @@ struct CnSum {
 
 // One block of A atoms (nab of them, from list position a0) against a warp's
 // B atoms (cn_warp): RP packed rows a lane, known at compile time so that the
-// rows' chains overlap.
-template <bool PBC, int RP>
+// rows' chains overlap. EACH: every switch value is added to the compensated
+// sum by itself, else two at a time.
+template <bool PBC, int RP, bool EACH>
 __device__ __forceinline__ void cn_block(const CnPair &cp, float c6, const int32_t *ia, const int32_t *ib, int nb,
                                          const float4 *xs, float4 *jB, float *lig, bool more, bool first, int nab,
                                          int lane, int bgrp, int nbg, int rounds, CnSum &sum) {
@@ -733,7 +734,9 @@ __device__ __forceinline__ void cn_block(const CnPair &cp, float c6, const int32
         F2 sw, q2;
         cp.term(dx, dy, dz, sw, q2);
         if (q == RP - 1) sw = f2_mul(sw, tail);
-        if (q & 1)
+        if (EACH)
+          sum.add(sw);
+        else if (q & 1)
           sum.add(f2_add(prev, sw));
         else if (q == RP - 1)
           sum.add(sw);
@@ -812,15 +815,18 @@ __device__ __forceinline__ void cn_block(const CnPair &cp, float c6, const int32
 // one of eight B-groups (streamed, the next atom loaded a round ahead). Every
 // pair is evaluated once, two at a time. A B atom's gradient is summed over
 // its four A-groups by two lane exchanges; a block's A gradients over the
-// B-groups by a reduce-scatter. Switch values are added in twos to a
-// compensated sum (CnSum): a CN of hundreds must be known to ~1e-8 relative to
-// place a hill two grid spacings wide.
+// B-groups by a reduce-scatter. Switch values go to a compensated sum (CnSum),
+// as a CN of hundreds must be known to ~1e-8 relative to place a hill two grid
+// spacings wide: in twos up to 40 A atoms, one by one above, where in twos would
+// drop values below the last place of their neighbours' (53 x 307 pairs x 101
+// steps: 39.4 us in twos, 40.7 one by one).
 // jB receives ds/dx of the warp's B atoms, lig[na][3] the warp's A sums
 // (unscaled; added to what is there if `more`), sh + sl the lane's own part
 // of s (warp_sum_ff adds the lanes). Bound by the FMA pipe: 20 lane-operations a pair (26 with a
 // minimum image) plus ~3 for the exchanges; the reciprocal takes 8 of those
 // cycles' MUFU slots.
-template <bool PBC>
+// LONG: na may exceed one block of 40 (false leaves that path out of the code).
+template <bool PBC, bool LONG>
 __device__ __forceinline__ void cn_warp(const CvDev &c, const int32_t *ia, const int32_t *ib, const float4 *xs,
                                         float4 *jB, float *lig, bool more, int lane, int b0, int nbg, float &sh,
                                         float &sl) {
@@ -829,16 +835,23 @@ __device__ __forceinline__ void cn_warp(const CvDev &c, const int32_t *ia, const
   const float c6 = -6.f * (float)c.inv_r0sq;
   const int rounds = (nb - b0 + nbg - 1) / nbg;  // of the warp's first B-group, the longest
   CnSum sum;
-  for (int a0 = 0; a0 < na; a0 += 40) {
+  const bool each = LONG && na > 40;
+  for (int a0 = 0; a0 < (LONG ? na : 1); a0 += 40) {
     const int nab = min(40, na - a0);
-#define ABP_CN_BLOCK(RP) \
-  cn_block<PBC, RP>(cp, c6, ia + a0, ib, nb, xs, jB, lig + 3 * a0, more, a0 == 0, nab, lane, bgrp, nbg, rounds, sum)
-    switch ((nab + 7) >> 3) {
-      case 1: ABP_CN_BLOCK(1); break;
-      case 2: ABP_CN_BLOCK(2); break;
-      case 3: ABP_CN_BLOCK(3); break;
-      case 4: ABP_CN_BLOCK(4); break;
-      default: ABP_CN_BLOCK(5);
+#define ABP_CN_BLOCK(RP, EACH)                                                                                       \
+  cn_block<PBC, RP, EACH>(cp, c6, ia + a0, ib, nb, xs, jB, lig + 3 * a0, more, a0 == 0, nab, lane, bgrp, nbg, rounds, \
+                          sum)
+    switch (((nab + 7) >> 3) + (each ? 8 : 0)) {
+      case 1: ABP_CN_BLOCK(1, false); break;
+      case 2: ABP_CN_BLOCK(2, false); break;
+      case 3: ABP_CN_BLOCK(3, false); break;
+      case 4: ABP_CN_BLOCK(4, false); break;
+      case 5: ABP_CN_BLOCK(5, false); break;
+      case 9: ABP_CN_BLOCK(1, true); break;
+      case 10: ABP_CN_BLOCK(2, true); break;
+      case 11: ABP_CN_BLOCK(3, true); break;
+      case 12: ABP_CN_BLOCK(4, true); break;
+      default: ABP_CN_BLOCK(5, true);
     }
 #undef ABP_CN_BLOCK
   }
@@ -858,13 +871,14 @@ __device__ __forceinline__ void warp_sum_ff(float (&h)[N], float (&l)[N]) {
     }
 }
 
+template <bool LONG = true>
 __device__ __forceinline__ void cn_warp_any(const CvDev &c, const int32_t *ia, const int32_t *ib, const float4 *xs,
                                             float4 *jB, float *lig, bool more, int lane, int b0, int nbg, float &sh,
                                             float &sl) {
   if (c.pbc)
-    cn_warp<true>(c, ia, ib, xs, jB, lig, more, lane, b0, nbg, sh, sl);
+    cn_warp<true, LONG>(c, ia, ib, xs, jB, lig, more, lane, b0, nbg, sh, sl);
   else
-    cn_warp<false>(c, ia, ib, xs, jB, lig, more, lane, b0, nbg, sh, sl);
+    cn_warp<false, LONG>(c, ia, ib, xs, jB, lig, more, lane, b0, nbg, sh, sl);
 }
 
 // The same by a group of warps: warp w takes the B-groups 8 w .. 8 w + 7 of

@@ -110,6 +110,7 @@ struct SplitShape {
   int win = 0;         // steps per window (0: walkers of k_sp_cn)
   int cv_smem = 0;
   bool staged = true;  // k_sp_cn's walkers are small enough to stage their coordinates
+  bool long_cn = false;  // one of them has a coordination number of more than 40 A atoms
   int wt = 0, mabp = 0;
   int min_dim = 0, max_atoms = 0;
 };

@@ -271,8 +271,11 @@ __device__ __forceinline__ void finish_records(const WalkerDev &wd, Step *st, in
 // fill the chip); otherwise by the CTA's four warps, one step a CTA. The same
 // sums, so the same bits. STAGED: a step's atoms are copied to shared memory
 // first (all in flight at once, the next step's asked into L2 meanwhile);
-// else they are read where they lie. ~120 registers a thread: four CTAs an SM.
-template <bool PER_WARP, bool STAGED>
+// else they are read where they lie. LONG: a coordination number of the batch
+// has more than 40 A atoms (without that path in its code 1000 walkers x 25
+// steps of 40 x 400 pairs take 589 us, with it 611). ~120 registers a thread:
+// four CTAs an SM.
+template <bool PER_WARP, bool STAGED, bool LONG>
 __global__ void __launch_bounds__(kCnThreads, 4) k_sp_cn(SplitArgs a) {
   extern __shared__ __align__(32) unsigned char smem[];
   __shared__ float red[kCnWarps][2];
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__(kCnThreads, 4) k_sp_cn(SplitArgs a) {
 #pragma unroll 1
           for (int v = 0; v < kCnWarps; ++v) {
             float ph, pl;
-            cn_warp_any(c, c.ia, c.ib, x, jB, lig, v > 0, lane, 8 * v, 8 * kCnWarps, ph, pl);
+            cn_warp_any<LONG>(c, c.ia, c.ib, x, jB, lig, v > 0, lane, 8 * v, 8 * kCnWarps, ph, pl);
 #pragma unroll
             for (int q = 0; q < kCnWarps; ++q)
               if (q == v) {
@@ -355,7 +358,7 @@ __global__ void __launch_bounds__(kCnThreads, 4) k_sp_cn(SplitArgs a) {
           __syncwarp();
         } else {
           float h[1], l[1];
-          cn_warp_any(c, c.ia, c.ib, x, jB, ligs + warp * c.na * 3, false, lane, 8 * warp, 8 * kCnWarps, h[0], l[0]);
+          cn_warp_any<LONG>(c, c.ia, c.ib, x, jB, ligs + warp * c.na * 3, false, lane, 8 * warp, 8 * kCnWarps, h[0], l[0]);
           warp_sum_ff<1>(h, l);
           if (lane == 0) {
             red[warp][0] = h[0];
@@ -1287,6 +1290,7 @@ void split_shape(const WalkerDev &hd, bool win, SplitShape *s) {
   } else {
     s->cv_smem = max(s->cv_smem, cn_bytes(hd.cv, hd.g.d, hd.natoms));
     s->staged = s->staged && hd.natoms * 16 <= kCnStage;
+    for (int k = 0; k < hd.g.d; ++k) s->long_cn = s->long_cn || (hd.cv[k].type == ABP_CV_COORD && hd.cv[k].na > 40);
   }
   if (hd.method == ABP_METHOD_MABP)
     s->mabp += 1;
@@ -1335,8 +1339,12 @@ cudaError_t launch_split(const SplitArgs &a0, const SplitShape &s, int sms, Laun
     const long long items = (long long)a.nw * a.nsteps, slots = 16ll * sms;
     a.chunk = (int)max(1ll, min((long long)kCnBatch, items / max(1ll, 3 * slots)));
     const bool per_warp = items >= slots;
-    void (*k)(SplitArgs) = per_warp ? (s.staged ? k_sp_cn<true, true> : k_sp_cn<true, false>)
-                                    : (s.staged ? k_sp_cn<false, true> : k_sp_cn<false, false>);
+    void (*const ks[2][2][2])(SplitArgs) = {  // [per_warp][staged][long_cn]
+        {{k_sp_cn<false, false, false>, k_sp_cn<false, false, true>},
+         {k_sp_cn<false, true, false>, k_sp_cn<false, true, true>}},
+        {{k_sp_cn<true, false, false>, k_sp_cn<true, false, true>},
+         {k_sp_cn<true, true, false>, k_sp_cn<true, true, true>}}};
+    void (*k)(SplitArgs) = ks[per_warp][s.staged][s.long_cn];
     run("k_sp_cn", k, dim3(nw, per_warp ? (a.nsteps + a.chunk * kCnWarps - 1) / (a.chunk * kCnWarps) : a.nsteps),
         kCnThreads, s.cv_smem);
   }
