@@ -955,7 +955,7 @@ __global__ void __launch_bounds__(kLineThreads) k_md_line(MdRunArgs a, const dou
     // a5 and the move of coordinate q
     if (q < 3) {
       const double dv = dvs, dt = add_rn(dv, dUs), u = us[q];
-      const bool keep_f = ra.forces || t == ra.nsteps - 1;
+      const bool keep_f = ra.forces || (a.last && t == ra.nsteps - 1);
       int bad = 0;
       for (int i = lane; i < natoms; i += 32) {
         const int ne = i == lane ? ne0 : wd.acnt[i];
