@@ -1501,6 +1501,7 @@ abp_status abp_md_run(abp_ctx *ctx, abp_walker *const *walkers, int n, void *coo
           MdRunArgs b = a;
           b.r.step0 = step0 + t;
           b.r.nsteps = std::min(block, nsteps - t);
+          b.first = t == 0;
           b.last = t + block >= nsteps;
           if (forces_dev) b.r.forces = static_cast<unsigned char *>(forces_dev) + t * fstep;
           if (traj_dev) b.traj = static_cast<unsigned char *>(traj_dev) + t * tstep;

@@ -187,7 +187,7 @@ struct MdRunArgs {
   void *traj;               // NULL: not recorded
   const long long *toff;
   long long tstride;
-  int last;                 // k_md_line: the call's last block of steps
+  int first, last;          // k_md_line: the call's first and last block of steps
 };
 
 // Closed-loop form of walkers whose CVs a thread evaluates (abp_md.cu).

@@ -869,10 +869,11 @@ __global__ void __launch_bounds__(kLineThreads) k_md_line(MdRunArgs a, const dou
     __syncwarp();
     __syncthreads();
     if (bads[0] | bads[1] | bads[2]) {
-      // this walker stops here: its state says so, its atoms stay
+      // this walker stops here: its state says so, its atoms stay (counted once
+      // a call, in the block of steps where it stops)
       if (tid == 0) {
+        if (a.first || !(wd.state->flags & ABP_WFLAG_NONFINITE)) atomicAdd(&ra.ctr->nonfinite, 1);
         wd.state->flags = ABP_WFLAG_NONFINITE;
-        atomicAdd(&ra.ctr->nonfinite, 1);
       }
       stopped = true;
       break;

@@ -1,8 +1,8 @@
 """FP64 closed loops of one COM distance in several blocks of steps (the noise
-of a block fits 64 MB): coordinates, trajectories, forces, grids and states as
-from one launch over all steps (a captured call). One walker starts with a
-non-finite atom, one stops in the second block, where its first hill is so high
-that it throws the atoms out of range."""
+of a block fits 64 MB): coordinates, trajectories, forces, grids, states and
+the count of stopped walkers as from one launch over all steps (a captured
+call). One walker starts with a non-finite atom, one stops in the second block,
+where its first hill is so high that it throws the atoms out of range."""
 import numpy as np
 import pytest
 import torch
@@ -87,4 +87,5 @@ def test_blocks_of_steps_equal_one_launch(record):
     for u, v in zip(a[1], b[1]):
         assert u["flags"] == v["flags"] and u["status"] == v["status"]
         assert u["V"] == v["V"] and np.array_equal(u["s"], v["s"]) and np.array_equal(u["dV"], v["dV"])
+    assert a[2] == b[2] and "1 walker steps" in a[2][0] and "2 walker steps" in a[2][1]
     assert [i for i, u in enumerate(a[1]) if u["flags"] & 8] == [3, 7]
