@@ -336,18 +336,27 @@ __device__ __forceinline__ int com_finish_ff(const CvDev &c, const float *ra, co
   return ABP_WFLAG_SINGULAR;
 }
 
-// An FP32 COM distance by one warp: every weighted offset from the group's
-// first atom formed exactly as hi + lo (the difference x - r_G split by
-// two_sum, the product's error by fma; the tiny w times the difference's low
-// part rounded once) and summed with two_sum per lane; group A's three sums
-// then on lanes 0-15 and group B's on lanes 16-31, where each exchange level
-// adds the partner's high part with its exact error going to the low part;
-// finished in hi + lo (com_finish_ff). A group of hundreds of atoms spread
-// over nanometres would otherwise lose ~1e-7 nm, several millionths of a hill
-// a few grid spacings wide. The result is lane 0's.
-__device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, const int32_t *ib, const float *wa,
-                                            const float *wb, const float4 *xs, int lane, float &s, float &sl,
-                                            float *u) {
+// Parts of an FP32 COM distance's sums: groups of more than kComWide atoms
+// together are summed in four parts (atoms i with i / 32 % 4 == v), taken by up
+// to four warps or one after another by one, and added in order: the same bits.
+// Several warps gain what three more lane exchanges cost one: 16 walkers x 25
+// steps in the form of one group each 262 -> 229 us at 2 x 520 atoms, 393 -> 301
+// at 2 x 1200 (128 threads in one sum: 285, 358); one walker's step by one warp
+// 14.3 -> 15.3 us and 21.2 -> 21.9. The line lies where one warp starts to lose
+// against 128 threads in one sum.
+constexpr int kComWide = 1280;
+__device__ __forceinline__ int com_parts(const CvDev &c) { return c.na + c.nb > kComWide ? 4 : 1; }
+
+// Part v of P by one warp: every weighted offset from the group's first atom
+// formed exactly as hi + lo (the difference x - r_G split by two_sum, the
+// product's error by fma; the tiny w times the difference's low part rounded
+// once) and summed with two_sum per lane; group A's three sums then on lanes
+// 0-15 and group B's on lanes 16-31, where each exchange level adds the
+// partner's high part with its exact error going to the low part. Lane 0 gets
+// A's sums, lane 16 B's.
+__device__ __forceinline__ void com_warp_part(const CvDev &c, const int32_t *ia, const int32_t *ib, const float *wa,
+                                              const float *wb, const float4 *xs, int lane, int v, int P,
+                                              float (&vh)[3], float (&vl)[3]) {
   const float4 ra = xs[ia[0]], rb = xs[ib[0]];
   float h[6] = {0, 0, 0, 0, 0, 0}, l[6] = {0, 0, 0, 0, 0, 0};
   auto acc = [&](int q, float w, float x, float r) {
@@ -360,14 +369,14 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
     h[q] = t;
     l[q] = __fadd_rn(l[q], __fadd_rn(e, pl));
   };
-  for (int i = lane; i < c.na; i += 32) {
+  for (int i = lane + 32 * v; i < c.na; i += 32 * P) {
     const float w = wa[i];
     const float4 p = xs[ia[i]];
     acc(0, w, p.x, ra.x);
     acc(1, w, p.y, ra.y);
     acc(2, w, p.z, ra.z);
   }
-  for (int i = lane; i < c.nb; i += 32) {
+  for (int i = lane + 32 * v; i < c.nb; i += 32 * P) {
     const float w = wb[i];
     const float4 p = xs[ib[i]];
     acc(3, w, p.x, rb.x);
@@ -375,7 +384,6 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
     acc(5, w, p.z, rb.z);
   }
   const bool up = (lane & 16) != 0;
-  float vh[3], vl[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     vh[q] = up ? h[3 + q] : h[q];
@@ -397,6 +405,35 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
       vh[q] = t;
       vl[q] = __fadd_rn(__fadd_rn(vl[q], ol), e);
     }
+}
+
+// A part's three sums (ph + pl) added to the parts' before it.
+__device__ __forceinline__ void com_add_part(float (&h)[3], float (&l)[3], const float *ph, const float *pl) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    float t, e;
+    two_sum<float>(h[q], ph[q], t, e);
+    h[q] = t;
+    l[q] = __fadd_rn(__fadd_rn(l[q], pl[q]), e);
+  }
+}
+
+// The COM distance by one warp (com_warp_part, the parts in order), finished in
+// hi + lo (com_finish_ff). A group of hundreds of atoms spread over nanometres
+// would otherwise lose ~1e-7 nm, several millionths of a hill a few grid
+// spacings wide. The result is lane 0's.
+__device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, const int32_t *ib, const float *wa,
+                                            const float *wb, const float4 *xs, int lane, float &s, float &sl,
+                                            float *u) {
+  const int P = com_parts(c);
+  float vh[3], vl[3];
+  com_warp_part(c, ia, ib, wa, wb, xs, lane, 0, P, vh, vl);
+#pragma unroll 1
+  for (int v = 1; v < P; ++v) {
+    float ph[3], pl[3];
+    com_warp_part(c, ia, ib, wa, wb, xs, lane, v, P, ph, pl);
+    com_add_part(vh, vl, ph, pl);
+  }
   float bh[3], bl[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -404,6 +441,7 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
     bl[q] = __shfl_sync(0xffffffffu, vl[q], 16);
   }
   if (lane != 0) return 0;
+  const float4 ra = xs[ia[0]], rb = xs[ib[0]];
   const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
   return com_finish_ff(c, a0, vh, vl, b0, bh, bl, s, sl, u);
 }
@@ -412,13 +450,51 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
 // group's weighted sum runs over offsets from the group's first atom, which
 // keeps the rounding at the scale of the group's extent rather than of the
 // absolute coordinates: R_G = r_G + sum_i w_i (x_i - r_G), sum_i w_i = 1.
-// FP32 walkers: by the group's first warp (com_one_warp).
+// FP32 walkers: by the group's first warp (com_one_warp), or the parts of a
+// wide one over its warps.
 template <typename Real>
 __device__ void cv_com(const Grp &g, GroupFixed<Real> *fx, int k, const typename Rec4<Real>::T *xs) {
   const CvDev &c = fx->wd.cv[k];
   const int32_t *ia = fx->ia[k], *ib = fx->ib[k];
   const Real *wa = fx->wa[k], *wb = fx->wb[k];
   if constexpr (sizeof(Real) == 4) {
+    const int P = com_parts(c);
+    if (P > 1 && g.nwarps > 1) {
+      float(*part)[2][6] = reinterpret_cast<float(*)[2][6]>(fx->red);  // [part][A, B][3 high, 3 low]
+      static_assert(sizeof(fx->red) >= 4 * 12 * sizeof(float), "the parts' sums fit red");
+      g.sync();  // red is free
+      for (int v = g.warp; v < P; v += g.nwarps) {
+        float vh[3], vl[3];
+        com_warp_part(c, ia, ib, wa, wb, xs, g.lane, v, P, vh, vl);
+        if ((g.lane & 15) == 0)
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            part[v][g.lane >> 4][q] = vh[q];
+            part[v][g.lane >> 4][3 + q] = vl[q];
+          }
+      }
+      g.sync();
+      if (g.t == 0) {
+        float h[2][3], l[2][3];
+#pragma unroll
+        for (int gr = 0; gr < 2; ++gr) {
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            h[gr][q] = part[0][gr][q];
+            l[gr][q] = part[0][gr][3 + q];
+          }
+          for (int v = 1; v < P; ++v) com_add_part(h[gr], l[gr], part[v][gr], part[v][gr] + 3);
+        }
+        const float4 ra = xs[ia[0]], rb = xs[ib[0]];
+        const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
+        float s = 0.f, sl = 0.f;
+        const int fl = com_finish_ff(c, a0, h[0], l[0], b0, h[1], l[1], s, sl, fx->com_u[k]);
+        fx->sh[k] = s;
+        fx->sl[k] = sl;
+        if (fl) atomicOr(&fx->flags, fl);
+      }
+      return;
+    }
     if (g.warp == 0) {
       float s = 0.f, sl = 0.f;
       const int fl = com_one_warp(c, ia, ib, wa, wb, xs, g.lane, s, sl, fx->com_u[k]);
