@@ -1269,8 +1269,10 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     if (lw.empty()) continue;
     RunArgs a{};
     if ((st = sub_table(ctx, lw, li, &a.table))) return st;
-    // unless a launch-shape knob asks for a group per walker (the same bits):
-    // short calls in one launch of the split form's parts, long ones in three
+    // unless a launch-shape knob asks for a group per walker (the same bits at
+    // the default width; another width adds a coordination number's parts in
+    // another order): short calls in one launch of the split form's parts, long
+    // ones in three
     bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1;
     bool mabp = false;
     for (size_t i = 0; split && i < lw.size(); ++i) {

@@ -22,8 +22,9 @@
 //
 // run over step records (StepRec) kept in a scratch block of the call, so the
 // parts without a chain use the whole chip however few walkers there are. The
-// arithmetic per step is the windowed form's (abp_window_ops.cuh): the same
-// bits, whichever form a call takes. FP32 grids.
+// arithmetic per step is the windowed form's (abp_window_ops.cuh), and a
+// coordination number's sum that of a group of 128 threads: the same bits as
+// the forms with a group per walker at their default width. FP32 grids.
 //
 // One group per walker against this form (GB300, whole calls): 3 walkers x 101
 // steps, 53 x 307 pairs, 4.04 ms -> 40 us; 1000 walkers x 25 steps, 40 x 400
