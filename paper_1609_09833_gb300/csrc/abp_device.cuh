@@ -183,10 +183,9 @@ __device__ __forceinline__ bool grp_any(const Grp &g, GroupFixed<Real> *fx, int 
   return r != 0;
 }
 
-template <typename Real, bool RN = false>
+template <typename Real>
 __device__ __forceinline__ Real min_image(Real dx, double box, double inv_box) {
-  if constexpr (RN) return fma_rn(-(Real)box, floor(fma_rn(dx, (Real)inv_box, (Real)0.5)), dx);
-  return dx - (Real)box * floor(dx * (Real)inv_box + (Real)0.5);
+  return fma_rn(-(Real)box, floor(fma_rn(dx, (Real)inv_box, (Real)0.5)), dx);
 }
 
 template <typename Real>
@@ -542,22 +541,15 @@ __device__ void cv_com(const Grp &g, GroupFixed<Real> *fx, int k, const typename
   }
 }
 
-template <typename Real, bool RN = false>
+template <typename Real>
 __device__ __forceinline__ void cross3(const Real *a, const Real *b, Real *o) {
-  if constexpr (RN) {
-    o[0] = fma_rn(a[1], b[2], -mul_rn(a[2], b[1]));
-    o[1] = fma_rn(a[2], b[0], -mul_rn(a[0], b[2]));
-    o[2] = fma_rn(a[0], b[1], -mul_rn(a[1], b[0]));
-  } else {
-    o[0] = a[1] * b[2] - a[2] * b[1];
-    o[1] = a[2] * b[0] - a[0] * b[2];
-    o[2] = a[0] * b[1] - a[1] * b[0];
-  }
+  o[0] = fma_rn(a[1], b[2], -mul_rn(a[2], b[1]));
+  o[1] = fma_rn(a[2], b[0], -mul_rn(a[0], b[2]));
+  o[2] = fma_rn(a[0], b[1], -mul_rn(a[1], b[0]));
 }
-template <typename Real, bool RN = false>
+template <typename Real>
 __device__ __forceinline__ Real dot3(const Real *a, const Real *b) {
-  if constexpr (RN) return fma_rn(a[2], b[2], fma_rn(a[0], b[0], mul_rn(a[1], b[1])));
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+  return fma_rn(a[2], b[2], fma_rn(a[0], b[0], mul_rn(a[1], b[1])));
 }
 
 // The dihedral angle of FP32 coordinates formed in FP64 (the coordinates
@@ -584,11 +576,10 @@ __device__ __forceinline__ double dihedral_angle64(const CvDev &c, const float (
 // Dihedral of atoms 1-2-3-4 at positions x: phi = atan2(|b2| b1.(b2 x b3),
 // (b1 x b2).(b2 x b3)), gradient in the Blondel-Karplus form, by one thread.
 // phi_lo receives the low part of the angle: 0, or with c.hp (FP32 walkers)
-// the FP64 angle's remainder after its FP32 rounding phi. RN: every product
-// and sum rounded as written (fma where written), so that each kernel's copy
-// computes the same bits; otherwise contraction is the compiler's (which, in
-// the closed-loop kernel, forms the same products: the bits agree).
-template <typename Real, bool RN = false>
+// the FP64 angle's remainder after its FP32 rounding phi. Every product and sum
+// is rounded as written (fma where written), so that each kernel's copy computes
+// the same bits.
+template <typename Real>
 __device__ __forceinline__ int dihedral_core(const CvDev &c, const Real (&x)[4][3], Real &phi, Real (*grad)[3],
                                              Real &phi_lo) {
   phi_lo = 0;
@@ -598,14 +589,14 @@ __device__ __forceinline__ int dihedral_core(const CvDev &c, const Real (&x)[4][
     b2[q] = x[2][q] - x[1][q];
     b3[q] = x[3][q] - x[2][q];
     if (c.pbc) {
-      b1[q] = min_image<Real, RN>(b1[q], c.box[q], c.inv_box[q]);
-      b2[q] = min_image<Real, RN>(b2[q], c.box[q], c.inv_box[q]);
-      b3[q] = min_image<Real, RN>(b3[q], c.box[q], c.inv_box[q]);
+      b1[q] = min_image<Real>(b1[q], c.box[q], c.inv_box[q]);
+      b2[q] = min_image<Real>(b2[q], c.box[q], c.inv_box[q]);
+      b3[q] = min_image<Real>(b3[q], c.box[q], c.inv_box[q]);
     }
   }
-  cross3<Real, RN>(b1, b2, m);
-  cross3<Real, RN>(b2, b3, n);
-  Real b2sq = dot3<Real, RN>(b2, b2);
+  cross3<Real>(b1, b2, m);
+  cross3<Real>(b2, b3, n);
+  Real b2sq = dot3<Real>(b2, b2);
   Real lb2 = sqrt(b2sq);
   if constexpr (sizeof(Real) == 4) {
     if (c.hp) {
@@ -613,37 +604,32 @@ __device__ __forceinline__ int dihedral_core(const CvDev &c, const Real (&x)[4][
       phi = (float)p64;
       phi_lo = (float)(p64 - (double)phi);
     } else {
-      phi = atan2(lb2 * dot3<Real, RN>(b1, n), dot3<Real, RN>(m, n));
+      phi = atan2(lb2 * dot3<Real>(b1, n), dot3<Real>(m, n));
     }
   } else {
-    phi = atan2(lb2 * dot3<Real, RN>(b1, n), dot3<Real, RN>(m, n));
+    phi = atan2(lb2 * dot3<Real>(b1, n), dot3<Real>(m, n));
   }
-  Real mm = dot3<Real, RN>(m, m), nn = dot3<Real, RN>(n, n);
+  Real mm = dot3<Real>(m, m), nn = dot3<Real>(n, n);
   if (!(mm > 0) || !(nn > 0) || !(lb2 > 0)) {
     for (int a = 0; a < 4; ++a)
       for (int q = 0; q < 3; ++q) grad[a][q] = 0;
     return ABP_WFLAG_SINGULAR;
   }
   Real inv_b2sq = rcp_fast<Real>(b2sq);
-  Real p = dot3<Real, RN>(b1, b2) * inv_b2sq, r = dot3<Real, RN>(b3, b2) * inv_b2sq;
+  Real p = dot3<Real>(b1, b2) * inv_b2sq, r = dot3<Real>(b3, b2) * inv_b2sq;
   Real cm = -lb2 * rcp_fast<Real>(mm), cn = lb2 * rcp_fast<Real>(nn);
   for (int q = 0; q < 3; ++q) {
     Real g1 = cm * m[q];
     Real g4 = cn * n[q];
     grad[0][q] = g1;
     grad[3][q] = g4;
-    if constexpr (RN) {
-      grad[1][q] = fma_rn(r, g4, -mul_rn(add_rn((Real)1, p), g1));
-      grad[2][q] = fma_rn(p, g1, -mul_rn(add_rn((Real)1, r), g4));
-    } else {
-      grad[1][q] = -(1 + p) * g1 + r * g4;
-      grad[2][q] = -(1 + r) * g4 + p * g1;
-    }
+    grad[1][q] = fma_rn(r, g4, -mul_rn(add_rn((Real)1, p), g1));
+    grad[2][q] = fma_rn(p, g1, -mul_rn(add_rn((Real)1, r), g4));
   }
   return 0;
 }
 
-// The dihedral of the atoms ia[0..3] of xs (dihedral_core, rounded as written).
+// The dihedral of the atoms ia[0..3] of xs (dihedral_core).
 template <typename Real>
 __device__ __forceinline__ int dihedral_eval(const CvDev &c, const int32_t *ia, const typename Rec4<Real>::T *xs,
                                              Real &phi, Real (*grad)[3], Real &phi_lo) {
@@ -655,7 +641,7 @@ __device__ __forceinline__ int dihedral_eval(const CvDev &c, const int32_t *ia, 
     x[a][1] = p.y;
     x[a][2] = p.z;
   }
-  return dihedral_core<Real, true>(c, x, phi, grad, phi_lo);
+  return dihedral_core<Real>(c, x, phi, grad, phi_lo);
 }
 
 template <typename Real>

@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(kLineThreads) k_md_line(MdRunArgs a, const dou
       const double hb = __shfl_sync(0xffffffffu, h, 16), pb = __shfl_sync(0xffffffffu, p0, 16);
       if (lane == 0) {
         double d = add_rn(sub_rn(pb, p0), sub_rn(hb, h));
-        if (c.pbc) d = min_image<double, true>(d, c.box[q], c.inv_box[q]);
+        if (c.pbc) d = min_image<double>(d, c.box[q], c.inv_box[q]);
         ds[q] = d;
       }
     }
