@@ -974,7 +974,7 @@ __device__ __forceinline__ void cv_coord_f32(const Grp &g, const CvDev &c, const
   g.sync();
 }
 
-// Coordination number for a group A of at most 4 * MAXA atoms, tiled over
+// FP64 coordination number for a group A of at most 4 * MAXA atoms, tiled over
 // the group's threads: lane & 3 picks one of four A-groups (A atoms i with
 // i % 4 == lane & 3, held in registers with their gradients) and t >> 2 one
 // of G/4 B-groups (B atoms j with j % (G/4) == t >> 2, streamed). Every pair
@@ -1090,22 +1090,12 @@ __device__ void cv_coord_tiled(const Grp &g, GroupFixed<Real> *fx, int k, const 
   }
 }
 
+// The same for longer groups A: thread t owns B entries t, t + G, ... (JB a
+// pass, gradients in registers); A entries in blocks of 4, their gradients
+// reduced over the warp, then summed over warps in a fixed order.
 template <typename Real>
-__device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typename Rec4<Real>::T *xs,
-                         typename Rec4<Real>::T *jA, typename Rec4<Real>::T *jB, Real *lig) {
-  if constexpr (sizeof(Real) == 4) {
-    float sh, sl;
-    cv_coord_f32(g, fx->wd.cv[k], fx->ia[k], fx->ib[k], xs, jA, jB, lig, fx->red, sh, sl);
-    if (g.t == 0) {
-      fx->sh[k] = sh;
-      fx->sl[k] = sl;
-    }
-    return;
-  } else {
-  if (fx->wd.cv[k].na <= 4 * 10) {
-    cv_coord_tiled<Real, 10>(g, fx, k, xs, jA, jB, lig);
-    return;
-  }
+__device__ void cv_coord_long(const Grp &g, GroupFixed<Real> *fx, int k, const typename Rec4<Real>::T *xs,
+                              typename Rec4<Real>::T *jA, typename Rec4<Real>::T *jB, Real *lig) {
   using R4 = typename Rec4<Real>::T;
   const CvDev &c = fx->wd.cv[k];
   const int32_t *ia = fx->ia[k], *ib = fx->ib[k];
@@ -1117,10 +1107,8 @@ __device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typena
   Real *mylig = lig + g.warp * c.na * 3;
   for (int q = g.lane; q < c.na * 3; q += 32) mylig[q] = 0;
   __syncwarp();
-  // this thread's partial sums, compensated (two-sum per term): a CN of
-  // thousands must be exact to ~1e-8 relative to place a hill two grid
-  // spacings wide, below FP32's resolution. One accumulator per owned B
-  // entry keeps the two-sum chains independent.
+  // this thread's partial sums, one compensated accumulator per owned B entry
+  // (independent two-sum chains)
   constexpr int JB = 4;
   Real sacc[JB], scomp[JB];
 #pragma unroll
@@ -1187,9 +1175,7 @@ __device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typena
       if (j < c.nb) jB[j] = make_rec<Real>(gxj[jj], gyj[jj], gzj[jj], (Real)0);
     }
   }
-  // the per-thread partial sums are combined in hi + lo arithmetic: a CN of
-  // a few hundred needs more than FP32's 24 bits to place a hill two grid
-  // spacings wide
+  // combined over the threads as hi + lo
   Real sh, sl;
   two_sum<Real>(sacc[0], scomp[0], sh, sl);
 #pragma unroll
@@ -1210,6 +1196,23 @@ __device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typena
     }
     jA[i] = make_rec<Real>(a0, a1, a2, (Real)0);
   }
+}
+
+// jA / jB receive ds/dx per list entry, lig is [warps][na][3] scratch.
+template <typename Real>
+__device__ void cv_coord(const Grp &g, GroupFixed<Real> *fx, int k, const typename Rec4<Real>::T *xs,
+                         typename Rec4<Real>::T *jA, typename Rec4<Real>::T *jB, Real *lig) {
+  if constexpr (sizeof(Real) == 4) {
+    float sh, sl;
+    cv_coord_f32(g, fx->wd.cv[k], fx->ia[k], fx->ib[k], xs, jA, jB, lig, fx->red, sh, sl);
+    if (g.t == 0) {
+      fx->sh[k] = sh;
+      fx->sl[k] = sl;
+    }
+  } else if (fx->wd.cv[k].na <= 4 * 10) {
+    cv_coord_tiled<Real, 10>(g, fx, k, xs, jA, jB, lig);
+  } else {
+    cv_coord_long<Real>(g, fx, k, xs, jA, jB, lig);
   }
 }
 
