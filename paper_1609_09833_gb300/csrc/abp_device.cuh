@@ -655,8 +655,10 @@ __device__ void cv_dihedral(const Grp &g, GroupFixed<Real> *fx, int k, const typ
 }
 
 // Two FP32 values in one 64-bit register: the packed FP32 instructions of
-// sm_100 and later (each half rounded as the scalar instruction rounds it).
-// They run at the scalar FMA rate per lane with half the issue slots.
+// sm_100 and later (each half rounded as the scalar instruction rounds it):
+// half the issue slots of scalar ones. Lane-operations a clock and SM, measured:
+// 51 with three different register pairs, 86 with a shared operand (scalar FMA
+// 85 and 116).
 using F2 = unsigned long long;
 __device__ __forceinline__ F2 f2_pack(float lo, float hi) {
   F2 r;
@@ -884,9 +886,10 @@ __device__ __forceinline__ void cn_block(const CnPair &cp, float c6, const int32
 // steps: 39.4 us in twos, 40.7 one by one).
 // jB receives ds/dx of the warp's B atoms, lig[na][3] the warp's A sums
 // (unscaled; added to what is there if `more`), sh + sl the lane's own part
-// of s (warp_sum_ff adds the lanes). Bound by the FMA pipe: 20 lane-operations a pair (26 with a
-// minimum image) plus ~3 for the exchanges; the reciprocal takes 8 of those
-// cycles' MUFU slots.
+// of s (warp_sum_ff adds the lanes). 20 lane-operations a pair (26 with a minimum
+// image), 18 cycles of the FMA pipe for a warp's 32 pairs; measured 38-40 cycles
+// of an SM quarter at any occupancy: packed instructions with three different
+// register pairs take longer to read them than to execute (F2).
 // LONG: na may exceed one block of 40 (false leaves that path out of the code).
 template <bool PBC, bool LONG>
 __device__ __forceinline__ void cn_warp(const CvDev &c, const int32_t *ia, const int32_t *ib, const float4 *xs,

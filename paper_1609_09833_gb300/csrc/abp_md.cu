@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(256, 1) k_md(MdRunArgs a) {
 // 2 the distance and the CV potential's gradient; the noise comes from a kernel
 // of its own on the other SMs (k_md_noise), scaled and read a step ahead. About
 // 40 FP64 instructions a step on the busiest warp against ~130 in k_md: one
-// walker of two 8-atom groups, 4.30 -> 2.3 us per step. The same
+// walker of two 8-atom groups, 4.30 -> 2.2 us per step. The same
 // operations in the same order as k_md, so the same bits.
 
 // The noise of steps [0, nsteps) of a block, c2 xi, as [walker][step][coordinate][atom].

@@ -27,9 +27,9 @@
 // the forms with a group per walker at their default width. FP32 grids.
 //
 // One group per walker against this form (GB300, whole calls): 3 walkers x 101
-// steps, 53 x 307 pairs, 4.04 ms -> 40 us; 1000 walkers x 25 steps, 40 x 400
-// pairs, 2.04 ms -> 0.61 ms; 64 walkers x 1000 steps of recorded frames 218
-// -> 146 us; two RMSDs with a 441-node hill every step 1.01 ms -> 176 us.
+// steps, 53 x 307 pairs, 4.04 ms -> 41 us; 1000 walkers x 25 steps, 40 x 400
+// pairs, 2.04 ms -> 0.59 ms; 64 walkers x 1000 steps of recorded frames 218
+// -> 154 us; two RMSDs with a 441-node hill every step 1.01 ms -> 176 us.
 #include <cuda_runtime.h>
 
 #include "abp_device.cuh"
@@ -273,9 +273,9 @@ __device__ __forceinline__ void finish_records(const WalkerDev &wd, Step *st, in
 // sums, so the same bits. STAGED: a step's atoms are copied to shared memory
 // first (all in flight at once, the next step's asked into L2 meanwhile);
 // else they are read where they lie. LONG: a coordination number of the batch
-// has more than 40 A atoms (without that path in its code 1000 walkers x 25
-// steps of 40 x 400 pairs take 589 us, with it 611). ~120 registers a thread:
-// four CTAs an SM.
+// has more than 40 A atoms. 1000 walkers x 25 steps of 40 x 400 pairs, whole
+// calls: 587 us staged without LONG, 611 with its path in the code, 614 not
+// staged. ~120 registers a thread: four CTAs an SM.
 template <bool PER_WARP, bool STAGED, bool LONG>
 __global__ void __launch_bounds__(kCnThreads, 4) k_sp_cn(SplitArgs a) {
   extern __shared__ __align__(32) unsigned char smem[];
