@@ -338,11 +338,11 @@ __device__ __forceinline__ int com_finish_ff(const CvDev &c, const float *ra, co
 // Parts of an FP32 COM distance's sums: groups of more than kComWide atoms
 // together are summed in four parts (atoms i with i / 32 % 4 == v), taken by up
 // to four warps or one after another by one, and added in order: the same bits.
-// Several warps gain what three more lane exchanges cost one: 16 walkers x 25
-// steps in the form of one group each 262 -> 229 us at 2 x 520 atoms, 393 -> 301
-// at 2 x 1200 (128 threads in one sum: 285, 358); one walker's step by one warp
-// 14.3 -> 15.3 us and 21.2 -> 21.9. The line lies where one warp starts to lose
-// against 128 threads in one sum.
+// 16 walkers x 25 steps in the form of one group each, us, at 2 x 520, 2 x 600
+// and 2 x 1200 atoms: by one warp 262, 273, 393; by 128 threads in one sum 285,
+// 289, 358; in four parts 307 at 2 x 1200. Where one warp has the whole distance
+// the parts cost three more lane exchanges (one walker's step 21.2 -> 21.9), so
+// the line lies where one warp starts to lose against one sum.
 constexpr int kComWide = 1280;
 __device__ __forceinline__ int com_parts(const CvDev &c) { return c.na + c.nb > kComWide ? 4 : 1; }
 
@@ -425,13 +425,12 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
                                             const float *wb, const float4 *xs, int lane, float &s, float &sl,
                                             float *u) {
   const int P = com_parts(c);
-  float vh[3], vl[3];
-  com_warp_part(c, ia, ib, wa, wb, xs, lane, 0, P, vh, vl);
+  float vh[3] = {0.f, 0.f, 0.f}, vl[3] = {0.f, 0.f, 0.f};
 #pragma unroll 1
-  for (int v = 1; v < P; ++v) {
+  for (int v = 0; v < P; ++v) {
     float ph[3], pl[3];
     com_warp_part(c, ia, ib, wa, wb, xs, lane, v, P, ph, pl);
-    com_add_part(vh, vl, ph, pl);
+    com_add_part(vh, vl, ph, pl);  // (to 0: the part as it is)
   }
   float bh[3], bl[3];
 #pragma unroll
@@ -443,6 +442,44 @@ __device__ __forceinline__ int com_one_warp(const CvDev &c, const int32_t *ia, c
   const float4 ra = xs[ia[0]], rb = xs[ib[0]];
   const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
   return com_finish_ff(c, a0, vh, vl, b0, bh, bl, s, sl, u);
+}
+
+// A wide COM distance over the warps of a group, for all its threads. Out of
+// line: inside the kernel's loop it slowed every other walker's step by 2-3 %.
+static __device__ __noinline__ void cv_com_wide(const Grp g, GroupFixed<float> *fx, int k, const float4 *xs) {
+  const CvDev &c = fx->wd.cv[k];
+  const int32_t *ia = fx->ia[k], *ib = fx->ib[k];
+  const float *wa = fx->wa[k], *wb = fx->wb[k];
+  const int P = com_parts(c);
+  float(*part)[2][6] = reinterpret_cast<float(*)[2][6]>(fx->red);  // [part][A, B][3 high, 3 low]
+  static_assert(sizeof(fx->red) >= 4 * 12 * sizeof(float), "the parts' sums fit red");
+  g.sync();  // red is free
+  for (int v = g.warp; v < P; v += g.nwarps) {
+    float vh[3], vl[3];
+    com_warp_part(c, ia, ib, wa, wb, xs, g.lane, v, P, vh, vl);
+    if ((g.lane & 15) == 0)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        part[v][g.lane >> 4][q] = vh[q];
+        part[v][g.lane >> 4][3 + q] = vl[q];
+      }
+  }
+  g.sync();
+  if (g.t != 0) return;
+  float h[2][3], l[2][3];
+#pragma unroll
+  for (int gr = 0; gr < 2; ++gr) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) h[gr][q] = l[gr][q] = 0.f;
+    for (int v = 0; v < P; ++v) com_add_part(h[gr], l[gr], part[v][gr], part[v][gr] + 3);
+  }
+  const float4 ra = xs[ia[0]], rb = xs[ib[0]];
+  const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
+  float s = 0.f, sl = 0.f;
+  const int fl = com_finish_ff(c, a0, h[0], l[0], b0, h[1], l[1], s, sl, fx->com_u[k]);
+  fx->sh[k] = s;
+  fx->sl[k] = sl;
+  if (fl) atomicOr(&fx->flags, fl);
 }
 
 // Centre-of-mass distance s = |R_B - R_A| (minimum image if pbc). Each
@@ -457,41 +494,8 @@ __device__ void cv_com(const Grp &g, GroupFixed<Real> *fx, int k, const typename
   const int32_t *ia = fx->ia[k], *ib = fx->ib[k];
   const Real *wa = fx->wa[k], *wb = fx->wb[k];
   if constexpr (sizeof(Real) == 4) {
-    const int P = com_parts(c);
-    if (P > 1 && g.nwarps > 1) {
-      float(*part)[2][6] = reinterpret_cast<float(*)[2][6]>(fx->red);  // [part][A, B][3 high, 3 low]
-      static_assert(sizeof(fx->red) >= 4 * 12 * sizeof(float), "the parts' sums fit red");
-      g.sync();  // red is free
-      for (int v = g.warp; v < P; v += g.nwarps) {
-        float vh[3], vl[3];
-        com_warp_part(c, ia, ib, wa, wb, xs, g.lane, v, P, vh, vl);
-        if ((g.lane & 15) == 0)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            part[v][g.lane >> 4][q] = vh[q];
-            part[v][g.lane >> 4][3 + q] = vl[q];
-          }
-      }
-      g.sync();
-      if (g.t == 0) {
-        float h[2][3], l[2][3];
-#pragma unroll
-        for (int gr = 0; gr < 2; ++gr) {
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            h[gr][q] = part[0][gr][q];
-            l[gr][q] = part[0][gr][3 + q];
-          }
-          for (int v = 1; v < P; ++v) com_add_part(h[gr], l[gr], part[v][gr], part[v][gr] + 3);
-        }
-        const float4 ra = xs[ia[0]], rb = xs[ib[0]];
-        const float a0[3] = {ra.x, ra.y, ra.z}, b0[3] = {rb.x, rb.y, rb.z};
-        float s = 0.f, sl = 0.f;
-        const int fl = com_finish_ff(c, a0, h[0], l[0], b0, h[1], l[1], s, sl, fx->com_u[k]);
-        fx->sh[k] = s;
-        fx->sl[k] = sl;
-        if (fl) atomicOr(&fx->flags, fl);
-      }
+    if (g.nwarps > 1 && com_parts(c) > 1) {
+      cv_com_wide(g, fx, k, xs);
       return;
     }
     if (g.warp == 0) {
