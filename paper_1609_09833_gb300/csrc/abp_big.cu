@@ -22,7 +22,7 @@
 // Each may start while the one before it ends (launch_chained). 32 walkers on a
 // shared 256^3 grid, 200 x 10,000 pairs each, 10 closed-loop steps: 1739 us
 // with a CTA per 1024 B entries (2.1 an SM), six launches a step and a look-up
-// per 256 atoms; 1136 us now, 91 us of a step's 113 in the pair kernel.
+// per 256 atoms; 1121 us now, 91 us of a step's 112 in the pair kernel.
 //
 // FP32_COMP grids only. The paper's bias routine is the serial counterpart
 // (one CPU rank), SI "Minimization of Interprocess Communications".
