@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -155,6 +156,7 @@ struct abp_ctx {
   unsigned long long use_clock = 0;
   int next_id = 0;
   int sms = 0;  // multiprocessors of the device
+  std::atomic<int> max_atoms{0};  // most atoms of a walker made in this context
   int tune_G = 0, tune_gpc = 0, tune_tile = -1;  // tile -1: library default (off; opt in with 1)
   int tune_lean = 0;
   std::vector<BigItem> big_key;                   // phased-form item lists of the last call
@@ -1029,6 +1031,7 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
   for (int k = 0; k < ncv; ++k)
     if (hd.cv[k].type == ABP_CV_COORD) pairs += (long long)hd.cv[k].na * hd.cv[k].nb;
   w->cost = pairs * 4 + d->natoms * 8 + stencil * 4 / d->stride;
+  if (d->natoms > ctx->max_atoms.load(std::memory_order_relaxed)) ctx->max_atoms = d->natoms;  // (under ctx->mu)
   *out = w;
   return ABP_OK;
 }
@@ -1233,7 +1236,8 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
   // a launch other threads may be storing another step's atom in the same
   // record, so every step gets launches of its own, which the stream orders
   // (a stride of 0 needs none of this: one thread keeps an atom's record).
-  if (forces && nsteps > 1 && fstride != 0) {
+  const int64_t most = ctx->max_atoms.load(std::memory_order_relaxed);  // (spares the walk over the list)
+  if (forces && nsteps > 1 && fstride != 0 && fstride > -most && fstride < most) {
     int64_t max_atoms = 0;
     for (int i = 0; i < n; ++i) max_atoms = std::max<int64_t>(max_atoms, walkers[i]->hd.natoms);
     if (fstride > -max_atoms && fstride < max_atoms) {
@@ -2055,7 +2059,6 @@ abp_status abp_sync(abp_ctx *ctx) {
 #include <functional>
 #include <memory>
 #include <thread>
-#include <atomic>
 #include <unordered_map>
 
 namespace {
