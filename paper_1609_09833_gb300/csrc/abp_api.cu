@@ -193,6 +193,7 @@ struct abp_walker {
   bool md_fast = false;
   bool md_line = false;  // FP64, well-tempered, one COM distance: k_md_line takes it
   long long cost = 0;  // rough work estimate used to order batched launches
+  long long pairs = 0;  // of its coordination numbers
 };
 
 namespace {
@@ -1030,6 +1031,7 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
   long long pairs = 0;
   for (int k = 0; k < ncv; ++k)
     if (hd.cv[k].type == ABP_CV_COORD) pairs += (long long)hd.cv[k].na * hd.cv[k].nb;
+  w->pairs = pairs;
   w->cost = pairs * 4 + d->natoms * 8 + stencil * 4 / d->stride;
   if (d->natoms > ctx->max_atoms.load(std::memory_order_relaxed)) ctx->max_atoms = d->natoms;  // (under ctx->mu)
   *out = w;
@@ -1206,6 +1208,22 @@ int short_max_steps(bool mabp) { return mabp ? 3 : 32; }
 int split_min_steps(int n, int sms, bool mabp) { return mabp ? 16 : n > sms ? 33 : 64; }
 constexpr int kShortSmem = 200 * 1024;  // shared memory of a short call's CTA, at most
 
+// Calls of a few steps over n walkers with coordination numbers (of `pairs`
+// pairs each on the average) that stay with a group per walker: the split
+// form's three launches cost ~20 us, again ~5 us past four step CTAs an SM,
+// a group per walker 4 to 11 us a step. Measured, us, split / group, pairs in
+// brackets: 1 step, 305 walkers 25 / 19 (100), 31 / 27 (2000), 34 / 29
+// (16,000), 1500 walkers 84 / 65, 98 / 79, 91 / 78; 2 steps, 16 walkers 22 / 16
+// (100), 28 / 23 (2000), 34 / 36 (16,000, two CVs), 500 walkers 34 / 31, 43 /
+// 45, 61 / 71; 3 steps, 16 walkers 22 / 20, 304 walkers 29 / 23 (100), 42 / 38
+// (6000), 305 walkers 32 / 38.
+bool cn_few_steps(int n, int sms, int nsteps, long long pairs) {
+  const bool one_round = n <= 2 * sms;  // of groups
+  if (nsteps == 1) return !one_round && pairs <= 16000;
+  if (nsteps == 2) return pairs < (one_round ? 16000 : 2000);
+  return nsteps == 3 && one_round && 3 * n > 4 * sms && pairs < 16000;
+}
+
 static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, const void *coords, int cdt,
                              const int64_t *coff, int64_t cstride, void *forces, const int64_t *foff,
                              int64_t fstride, int mode, int64_t step0, int nsteps) {
@@ -1278,8 +1296,11 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     // another order): short calls in one launch of the split form's parts, long
     // ones in three
     bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1;
-    bool mabp = false;
+    bool mabp = false, cn = !win;
+    long long pairs = 0;
     for (size_t i = 0; split && i < lw.size(); ++i) {
+      cn = cn && lw[i]->has_cn;
+      pairs += lw[i]->pairs;
       // (a walker whose group does not fit is refused below, whatever the form)
       split = lw[i]->group_fits && split_eligible(lw[i]->hd, win);
       mabp = mabp || lw[i]->hd.method == ABP_METHOD_MABP;
@@ -1310,7 +1331,7 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
           continue;
         }
       }
-      if (!win || nsteps >= split_min_steps(n, ctx->sms, mabp)) {
+      if (win ? nsteps >= split_min_steps(n, ctx->sms, mabp) : !(cn && cn_few_steps(n, ctx->sms, nsteps, pairs / n))) {
         bool done = false;
         if ((st = run_split(ctx, lw, a.table, win, s, nsteps, &done))) return st;
         if (done) continue;
