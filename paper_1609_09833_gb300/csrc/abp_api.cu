@@ -1511,14 +1511,17 @@ abp_status abp_md_run(abp_ctx *ctx, abp_walker *const *walkers, int n, void *coo
     bool fast = !fp64;
     for (abp_walker *w : lw) fast = fast && w->md_fast;
     // FP64 walkers of one COM distance, one an SM at most (more of them fill
-    // the FP64 pipes as it is), in blocks of steps whose noise fits the scratch
+    // the FP64 pipes as it is), in blocks of steps whose noise fits the scratch.
+    // One or two steps of small walkers are done before the second launch pays
+    // (us, k_md / line, 16, 60 and 250 atoms: 1 step 19 / 25, 19 / 22, 39 / 27; 2
+    // steps 23 / 25, 28 / 25, 66 / 33; 3 steps 27 / 24, 37 / 28, 77 / 40).
     bool line = fp64 && dim == 1 && (int)lw.size() <= ctx->sms;
     int max_atoms = 1;
     for (abp_walker *w : lw) {
       line = line && w->md_line;
       max_atoms = std::max(max_atoms, w->hd.natoms);
     }
-    if (line) {
+    if (line && (nsteps > 2 || nsteps * max_atoms >= 100)) {
       const size_t per_step = md_noise_bytes(a.r.nw, max_atoms, 1);
       const int block = (int)std::min<size_t>(nsteps, std::max<size_t>(1, kNoiseScratch / per_step));
       Scratch noise(ctx, per_step * block);

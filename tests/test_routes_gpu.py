@@ -66,3 +66,19 @@ def test_few_steps_of_coordination_numbers(nl, npk, n, T, want):
     group, ref = _call(abp, sp, nw, T, knob=128)
     assert group == GROUP
     _same(out, ref)
+
+
+@pytest.mark.parametrize("natoms,T,line", [(16, 1, False), (99, 1, False), (100, 1, True), (49, 2, False),
+                                           (50, 2, True), (16, 3, True)])
+def test_few_steps_of_an_fp64_closed_loop(natoms, T, line):
+    from paper_1609_09833_gb300 import abp
+
+    sp = {"natoms": natoms, "cvs": [{"type": "com_dist", "a": np.arange(natoms // 2), "b": np.arange(natoms // 2, natoms)}],
+          "grid": synth.grid((-2.0,), (4.0,), (512,), (False,)), "hill": synth.hill(0.8, (0.05,), 1, 8.0)}
+    names, out = _call(abp, sp, 3, T, fp64=True, md=True)
+    assert names == ({"k_md_noise", "k_md_line"} if line else {"k_md"})
+    many, ref = _call(abp, sp, _sms() + 1, T, fp64=True, md=True)  # (more than one walker an SM: k_md)
+    assert many == {"k_md"}
+    n = 1 * natoms  # every walker has its own atoms but the first ones are drawn alike
+    assert np.array_equal(out[0][:, :n], ref[0][:, :n]) and np.array_equal(out[1][:, :n], ref[1][:, :n])
+    assert out[1].any() and np.array_equal(out[2], ref[2])
