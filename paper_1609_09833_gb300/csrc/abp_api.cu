@@ -186,7 +186,9 @@ struct abp_walker {
   bool big = false;    // runs in the phased form (shared grid, or too large for a walker group)
   bool win = false;    // runs in the windowed form of the fused kernel (COM distance / dihedral CVs)
   bool has_rmsd = false;
-  bool group_fits = false;  // a walker group of the default width fits one SM's shared memory
+  // FP32: the split form and the short calls take it. Not if a group of the
+  // default width exceeds one SM's shared memory, which every form refuses.
+  bool split = false;
   // the closed-loop kernel's register-fed form applies: FP32 WT walkers of at
   // most 64 atoms of at most two a5 terms each, COM groups of at most 16
   // atoms, the other CVs dihedrals
@@ -936,8 +938,6 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
   // for one shared-memory walker group (FP32, at most one CN)
   w->big = grid->desc.shared || run_group_bytes(hd, fp64, 32, 0, false) > 227 * 1024;
   w->win = !w->big && window_eligible(hd, fp64);
-  w->group_fits = run_group_bytes(hd, fp64, w->win ? kWinGroup : w->has_cn ? kCnGroup : kRunGroup, 0, w->win) <=
-                  227 * 1024;
   if (w->win) {
     // the closed-loop form's a5 term tables (read, not rebuilt, by each launch)
     std::vector<int> tcnt;
@@ -1028,6 +1028,8 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
     delete w;
     return st;
   }
+  w->split = !fp64 && !w->big && split_eligible(hd, w->win) &&
+             run_group_bytes(hd, fp64, w->win ? kWinGroup : w->has_cn ? kCnGroup : kRunGroup, 0, w->win) <= 227 * 1024;
   long long pairs = 0;
   for (int k = 0; k < ncv; ++k)
     if (hd.cv[k].type == ABP_CV_COORD) pairs += (long long)hd.cv[k].na * hd.cv[k].nb;
@@ -1301,8 +1303,7 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     for (size_t i = 0; split && i < lw.size(); ++i) {
       cn = cn && lw[i]->has_cn;
       pairs += lw[i]->pairs;
-      // (a walker whose group does not fit is refused below, whatever the form)
-      split = lw[i]->group_fits && split_eligible(lw[i]->hd, win);
+      split = lw[i]->split;  // (if its group does not fit it is refused below)
       mabp = mabp || lw[i]->hd.method == ABP_METHOD_MABP;
     }
     if (split) {
