@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -189,6 +190,7 @@ struct abp_walker {
   // FP32: the split form and the short calls take it. Not if a group of the
   // default width exceeds one SM's shared memory, which every form refuses.
   bool split = false;
+  bool full_window = false;  // its coordinates allow windows of kWinMax steps
   // the closed-loop kernel's register-fed form applies: FP32 WT walkers of at
   // most 64 atoms of at most two a5 terms each, COM groups of at most 16
   // atoms, the other CVs dihedrals
@@ -1028,6 +1030,7 @@ abp_status abp_walker_create(abp_ctx *ctx, abp_grid *grid, const abp_walker_desc
     delete w;
     return st;
   }
+  w->full_window = w->win && window_steps(hd.natoms, hd.cv, ncv, rsz) == kWinMax;
   w->split = !fp64 && !w->big && split_eligible(hd, w->win) &&
              run_group_bytes(hd, fp64, w->win ? kWinGroup : w->has_cn ? kCnGroup : kRunGroup, 0, w->win) <= 227 * 1024;
   long long pairs = 0;
@@ -1205,9 +1208,19 @@ static abp_status run_split(abp_ctx *ctx, const std::vector<abp_walker *> &ws, c
 // ~16 us and then 0.2 us a step (well-tempered) or 1 us a step (mABP), each
 // again per round of walkers over the SMs: 64 walkers 32 steps 28 / 23, 64
 // steps 31 / 31, 256 steps 50 / 66; 300 walkers 32 steps 31 / 44; mABP 16
-// steps 27 / 29.
+// steps 27 / 29. Walkers of up to 63 atoms (windows of 32 steps) at most one an
+// SM, split / group: two CVs 64 steps 27 / 24 to 37 / 37, 100 steps 30 / 36 to
+// 42 / 46; one CV, whose stencil a group deposits in one round (~1.3 us a
+// deposit less), stride 100: 64 steps 28 / 22, 150 steps 29 / 27 to 32 / 36, 250
+// steps 33 / 37 to 36 / 53, stride 20: 100 steps 43 / 36, 400 steps 106 / 98 to
+// 111 / 106.
 int short_max_steps(bool mabp) { return mabp ? 3 : 32; }
-int split_min_steps(int n, int sms, bool mabp) { return mabp ? 16 : n > sms ? 33 : 64; }
+bool split_pays(int n, int sms, bool mabp, int d, bool full_window, double stride, int nsteps) {
+  if (mabp) return nsteps >= 16;
+  if (n > sms) return nsteps >= 33;
+  if (!full_window) return nsteps >= 64;
+  return d > 1 ? nsteps >= 80 : nsteps * (stride - 20) > 140 * stride;
+}
 constexpr int kShortSmem = 200 * 1024;  // shared memory of a short call's CTA, at most
 
 // Calls of a few steps over n walkers with coordination numbers (of `pairs`
@@ -1298,11 +1311,13 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
     // another order): short calls in one launch of the split form's parts, long
     // ones in three
     bool split = !fp64 && !ctx->tune_G && !ctx->tune_gpc && !ctx->tune_lean && ctx->tune_tile != 1;
-    bool mabp = false, cn = !win;
-    long long pairs = 0;
+    bool mabp = false, cn = !win, full_window = true;
+    long long pairs = 0, stride = LLONG_MAX;
     for (size_t i = 0; split && i < lw.size(); ++i) {
       cn = cn && lw[i]->has_cn;
       pairs += lw[i]->pairs;
+      full_window = full_window && lw[i]->full_window;
+      stride = std::min<long long>(stride, lw[i]->hd.stride);
       split = lw[i]->split;  // (if its group does not fit it is refused below)
       mabp = mabp || lw[i]->hd.method == ABP_METHOD_MABP;
     }
@@ -1332,7 +1347,8 @@ static abp_status run_common(abp_ctx *ctx, abp_walker *const *walkers, int n, co
           continue;
         }
       }
-      if (win ? nsteps >= split_min_steps(n, ctx->sms, mabp) : !(cn && cn_few_steps(n, ctx->sms, nsteps, pairs / n))) {
+      if (win ? split_pays(n, ctx->sms, mabp, form + 1, full_window, (double)stride, nsteps)
+              : !(cn && cn_few_steps(n, ctx->sms, nsteps, pairs / n))) {
         bool done = false;
         if ((st = run_split(ctx, lw, a.table, win, s, nsteps, &done))) return st;
         if (done) continue;

@@ -82,3 +82,23 @@ def test_few_steps_of_an_fp64_closed_loop(natoms, T, line):
     n = 1 * natoms  # every walker has its own atoms but the first ones are drawn alike
     assert np.array_equal(out[0][:, :n], ref[0][:, :n]) and np.array_equal(out[1][:, :n], ref[1][:, :n])
     assert out[1].any() and np.array_equal(out[2], ref[2])
+
+
+@pytest.mark.parametrize("natoms,d,stride,n,T,split", [
+    (40, 2, 20, 3, 79, False), (40, 2, 20, 3, 80, True), (40, 2, 100, "s+1", 33, True), (200, 2, 20, 3, 64, True),
+    (40, 1, 100, 3, 175, False), (40, 1, 100, 3, 176, True), (40, 1, 20, 3, 600, False), (40, 1, 1, 3, 300, False),
+    (40, 1, 1 << 40, 3, 141, True), (200, 1, 20, 3, 64, True), (40, 1, 20, "s+1", 33, True)])
+def test_long_calls_of_windowed_walkers(natoms, d, stride, n, T, split):
+    from paper_1609_09833_gb300 import abp
+
+    cvs = [{"type": "com_dist", "a": np.arange(natoms // 2), "b": np.arange(natoms // 2, natoms)},
+           {"type": "dihedral", "a": np.arange(4)}][:d]
+    g = synth.grid((0.0, -np.pi)[:d], (3.0, np.pi)[:d], (64, 64)[:d], (False, True)[:d])
+    sp = {"natoms": natoms, "cvs": cvs, "grid": g,
+          "hill": synth.hill(0.5, [synth.bins(g, k, 2.0) for k in range(d)], stride, 12.0)}
+    nw = _sms() + 1 if n == "s+1" else n
+    names, out = _call(abp, sp, nw, T)
+    assert names == ({"k_sp_cv", "k_sp_chain", "k_sp_force"} if split else {"k_win"})
+    group, ref = _call(abp, sp, nw, T, knob=256)
+    assert group == {"k_win"}
+    _same(out, ref)
