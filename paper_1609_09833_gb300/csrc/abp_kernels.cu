@@ -530,8 +530,12 @@ struct WindowCtx {
   // chain half's warps (23 x 23 nodes x 32 hills x ~40 on four warps). Two
   // RMSD CVs on 480 x 480, 441-node hills, 64 walkers x 1000 steps: 1.55 ms
   // with a box in shared memory and a barrier per hill, 1.01 ms now.
-  // Returns false (nothing done) for a union of more than kMabpUnion nodes:
-  // there the nodes no hill covers cost more than chain_seq's barriers.
+  // Returns false (nothing done) for a union of more than kMabpUnion nodes, or of
+  // more than 3/5 of a round of NB nodes a thread and a stencil for each of its
+  // hills (hills far apart): there the nodes no hill covers cost more than
+  // chain_seq, which takes about that for a hill. 3D, 729-node hills every other step at
+  // random places, 8 steps of 600 walkers: 350 us node by node, 206 hill by hill; along a
+  // slow path 127 and 148.
   template <int DIM>
   __device__ bool chain_mabp(const Grp &g, int w) const {
     const WalkerDev &wd = fx->wd;
@@ -576,7 +580,10 @@ struct WindowCtx {
         }
         nodes *= span[k];
       }
-      if (nodes > kMabpUnion) return false;
+      long long stencil = 1;
+#pragma unroll
+      for (int k = 0; k < d; ++k) stencil *= 2 * wd.R[k] + 1;
+      if (nodes > kMabpUnion || 5 * nodes > 3 * __popc(gdep) * (NB * g.G + stencil)) return false;
     }
     // is node j inside the union?
     auto inside = [&](const int *j) -> bool {
